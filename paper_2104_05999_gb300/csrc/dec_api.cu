@@ -127,6 +127,8 @@ dec_status dec_mesh_upload(dec_ctx* ctx, const double* xyz, int64_t n_nodes,
   ctx->n = n_nodes;
   ctx->m = n_tets;
   ctx->nf = 0;              // faces of the tet-centred form: rebuilt on demand
+  ctx->order_built = false;  // so are the spatial node order and the layouts over it
+  ctx->batch_form = -1;
   ctx->tet_solved = false;
   cudaStream_t s = ctx->stream;
   DEC_TRY(upload(ctx->xyz, xyz, 3 * n_nodes, s));

@@ -88,6 +88,7 @@ struct BatchArgs {
   double rtol2, seg2;
   int max_iter;
   int warm;                               // start from x64 (the last solution)
+  int spread;                             // fewer windows than blocks: see windows()
   double* phase;                          // [6] per-phase device time, block 0
   int64_t Ltotal, Gtotal[2];              // entries of the sliced layouts
 };
@@ -114,31 +115,25 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-__device__ __forceinline__ bool bgrid_sync(unsigned* bar, int* err) {
+// Grid barrier over a counter that only grows: `target` is the arrival count
+// that lets this round pass (the launch clears the counter).  Returns false
+// once any block has given up (then every block leaves at its next barrier).
+__device__ __forceinline__ bool bgrid_sync(unsigned* bar, int* err, unsigned& target) {
   __syncthreads();
+  target += gridDim.x;
   if (threadIdx.x == 0) {
-    volatile unsigned* gen = bar + 1;
-    const unsigned g = *gen;
     __threadfence();
-    const unsigned arrived = atomicAdd(bar, 1u);
-    if (arrived == gridDim.x - 1) {
-      bar[0] = 0u;
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      // bar[2] != 0 replaces the poll limit (the context's barrier test)
-      const unsigned lim = *(volatile unsigned*)(bar + 2);
-      const long limit = lim ? (long)lim : kBSpinLimit;
-      long polls = 0;
-      unsigned ns = 32;
-      while (*gen == g) {
-        if (++polls > limit || *(volatile int*)err) {
-          atomicExch(err, 1);
-          break;
-        }
-        __nanosleep(ns);
-        if (ns < 256) ns <<= 1;
+    atomicAdd(bar, 1u);
+    // bar[2] != 0 replaces the poll limit (the context's barrier test)
+    const unsigned lim = *(volatile unsigned*)(bar + 2);
+    const long limit = lim ? (long)lim : kBSpinLimit;
+    long polls = 0;
+    while ((int)(*(volatile unsigned*)bar - target) < 0) {
+      if (++polls > limit || *(volatile int*)err) {
+        atomicExch(err, 1);
+        break;
       }
+      if (polls > 16) __nanosleep(polls > 256 ? 256 : 20);
     }
     __threadfence();
   }
@@ -160,33 +155,70 @@ struct BState {
 };
 
 // Per-instance grid reduction; thread (r, q) of a warp contributes v[j] to
-// instance 4q + j.  Lanes of equal q are summed by shuffles, the 32 warps'
-// sums by one warp per instance, the blocks' partials by one warp per
-// instance after the grid barrier (lane l adds partials l, l + 32, ...), all
-// in a fixed order.  The result lands in S.red[b], identical in every block.
+// instance 4q + j.  The result lands in S.red[b], identical in every block:
+// lanes of equal q are summed by shuffles, then the 32 warps, then the
+// blocks' partials after the grid barrier, all in a fixed order.  GB300's
+// FP64 pipe adds one warp in 16 cycles, so each add is made to work on up to
+// 32 different sums: butterflies of all four values in every lane, and one
+// warp per instance over the blocks' partials, kept that pipe busy for 14 us
+// a reduction at 64 instances (3,375 nodes; 5 us now, and a batched solve of
+// 64 crack paths there 5.8 -> 2.9 ms with the spread slices below).
 __device__ bool breduce(const double (&v)[kIPT], const BatchArgs& a, int& parity, BState& S,
-                        double (*shw)[kBMax], int* err) {
+                        double (*shw)[kBMax], double (*sh4)[kBMax], int* err, unsigned& target) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int TPR = a.TPR, BS = a.BS, G = gridDim.x;
-#pragma unroll
-  for (int j = 0; j < kIPT; ++j) {
-    double x = v[j];
-    for (int o = 16; o >= TPR; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane < TPR) shw[warp][kIPT * lane + j] = x;
+  {  // each step halves the values a lane still sums
+    const int h16 = (lane >> 4) & 1, h8 = (lane >> 3) & 1;
+    double k0 = h16 ? v[2] : v[0], k1 = h16 ? v[3] : v[1];
+    k0 += __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16);
+    k1 += __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16);
+    if (TPR <= 8) {
+      double k = h8 ? k1 : k0;
+      k += __shfl_xor_sync(0xffffffffu, h8 ? k0 : k1, 8);
+      for (int o = 4; o >= TPR; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+      if ((lane & 7) < TPR) shw[warp][kIPT * (lane & 7) + 2 * h16 + h8] = k;
+    } else {
+      shw[warp][kIPT * (lane & 15) + 2 * h16] = k0;
+      shw[warp][kIPT * (lane & 15) + 2 * h16 + 1] = k1;
+    }
   }
   __syncthreads();
   double* part = a.partial + (size_t)parity * G * BS;
   parity ^= 1;
-  for (int b = warp; b < BS; b += kBWarps) {
-    const double x = warp_sum(shw[lane][b]);
-    if (lane == 0) part[(size_t)blockIdx.x * BS + b] = x;
-  }
-  if (!bgrid_sync(a.bar, err)) return false;
-  for (int b = warp; b < BS; b += kBWarps) {
+  const int i = threadIdx.x % BS;
+  if (threadIdx.x < 4 * BS) {        // the warps' sums, a quarter of the warps each
     double x = 0.0;
-    for (int blk = lane; blk < G; blk += 32) x += __ldcg(part + (size_t)blk * BS + b);
-    x = warp_sum(x);
-    if (lane == 0) S.red[b] = x;
+#pragma unroll
+    for (int w = 0; w < kBWarps / 4; ++w) x += shw[4 * w + threadIdx.x / BS][i];
+    sh4[threadIdx.x / BS][i] = x;
+  }
+  __syncthreads();
+  if (threadIdx.x < BS)
+    part[(size_t)blockIdx.x * BS + i] = (sh4[0][i] + sh4[1][i]) + (sh4[2][i] + sh4[3][i]);
+  if (!bgrid_sync(a.bar, err, target)) return false;
+  {  // the blocks' partials: thread (chunk, instance), then the chunks
+    double x = 0.0;
+    constexpr int U = 5;                           // partials in flight per thread
+    const int step = kBBlock / BS;
+    for (int c = threadIdx.x / BS; c < G; c += U * step) {
+      double y[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        y[u] = c + u * step < G ? __ldcg(part + (size_t)(c + u * step) * BS + i) : 0.0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) x += y[u];
+    }
+    for (int o = 16; o >= BS; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    const int per = BS < 32 ? 32 : BS;             // threads of a row of sums
+    if (BS >= 32 || lane < BS) shw[threadIdx.x / per][i] = x;
+    __syncthreads();
+    if (threadIdx.x < 4 * BS) {
+      double y = 0.0;
+      for (int c = threadIdx.x / BS; c < kBBlock / per; c += 4) y += shw[c][i];
+      sh4[threadIdx.x / BS][i] = y;
+    }
+    __syncthreads();
+    if (threadIdx.x < BS) S.red[i] = (sh4[0][i] + sh4[1][i]) + (sh4[2][i] + sh4[3][i]);
   }
   __syncthreads();
   return true;
@@ -504,6 +536,7 @@ pcg_batched_persistent(BatchArgs a) {
   if (*(volatile unsigned*)(a.bar + 3) && blockIdx.x == gridDim.x - 1) return;
   __shared__ BState S;
   __shared__ double shw[kBWarps][kBMax];
+  __shared__ double sh4[4][kBMax];
   const int BS = a.BS, TPR = a.TPR, C = a.C;
   const int64_t n = a.n;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -516,12 +549,22 @@ pcg_batched_persistent(BatchArgs a) {
   for (int j = 0; j < kIPT; ++j) st[j] = kIPT * q + j;
   int* err = a.status;
   int parity = 0;
+  unsigned target = 0;
   float4* X = reinterpret_cast<float4*>(a.x);
   float4* R = reinterpret_cast<float4*>(a.r);
   float4* Z = reinterpret_cast<float4*>(a.z);
   float4* Pv = reinterpret_cast<float4*>(a.p);
   float4* Q = reinterpret_cast<float4*>(a.q);
   float4* T = reinterpret_cast<float4*>(a.t);
+  auto count_flags = [&](const int* flags) {   // instances with a flag, into S.count
+    if (warp == 0) {
+      int c = 0;
+      for (int i = lane; i < BS; i += 32) c += flags[i];
+      c = __reduce_add_sync(0xffffffffu, c);
+      if (lane == 0) S.count = c;
+    }
+    __syncthreads();
+  };
   auto act = [&](const int* flags, int j) { return flags[kIPT * q + j] != 0; };
   auto any4 = [&](const int* flags) {
     return flags[kIPT * q] | flags[kIPT * q + 1] | flags[kIPT * q + 2] | flags[kIPT * q + 3];
@@ -539,7 +582,16 @@ pcg_batched_persistent(BatchArgs a) {
   // are sorted by length inside a window, so the warp-to-slice assignment
   // rotates by 13 (coprime to 32) from window to window: every warp gets
   // long and short slices alike instead of warp 0 always the longest.
+  // With fewer windows than blocks (small meshes) the slices are spread over
+  // all blocks instead, one per warp: slice warp * gridDim + block.  At 3,375
+  // nodes and 64 instances 53 of 152 SMs had work.
+  const int64_t spread_s = (int64_t)warp * gridDim.x + blockIdx.x;
+  const bool spread_on = spread_s < a.nwin * kBWarps;
   auto windows = [&](const int32_t* perm, auto&& body) {
+    if (a.spread) {
+      if (spread_on) body(spread_s, __ldg(perm + spread_s * C + r));
+      return;
+    }
     int k = 0;
     for (int64_t win = blockIdx.x; win < a.nwin; win += gridDim.x, ++k) {
       const int64_t s = win * kBWarps + ((warp + 13 * k) & (kBWarps - 1));
@@ -558,6 +610,13 @@ pcg_batched_persistent(BatchArgs a) {
   };
   auto windows_pf = [&](const int32_t* perm, const int32_t* sptr, auto&& pf_struct,
                         const float4* V0, const float4* V1, auto&& body) {
+    if (a.spread) {
+      if (spread_on) {
+        const int32_t b0 = __ldg(sptr + spread_s), b1 = __ldg(sptr + spread_s + 1);
+        body(b0, (b1 - b0) / C, __ldg(perm + spread_s * C + r));
+      }
+      return;
+    }
     int64_t win = blockIdx.x;
     if (win >= a.nwin) return;
     int k = 0;
@@ -621,7 +680,7 @@ pcg_batched_persistent(BatchArgs a) {
                     const float4* V0, const float4* V1, const char* A0, int eb0,
                     const char* A1, int eb1, auto&& consume, auto&& finish) {
     int64_t win = blockIdx.x;
-    if (win >= a.nwin) return;
+    if (a.spread ? !spread_on : win >= a.nwin) return;
     extern __shared__ __align__(16) float4 bsm_slots[];
     const int chunk = STAGE * C * (STAGE_L ? 8 : 6);
     char* wb = reinterpret_cast<char*>(bsm_slots) + (size_t)warp * 2 * chunk;
@@ -641,13 +700,13 @@ pcg_batched_persistent(BatchArgs a) {
     auto slice_of = [&](int64_t w, int kk) {
       return w * kBWarps + ((warp + 13 * kk) & (kBWarps - 1));
     };
-    int64_t s = slice_of(win, 0);
+    const int64_t s = a.spread ? spread_s : slice_of(win, 0);
     int32_t row = __ldg(perm + s * C + r), b0 = __ldg(sptr + s);
     int32_t W = (__ldg(sptr + s + 1) - b0) / C;
     int cb = 0;
     bool have = false;          // this slice's first chunk is already in buffer cb
     for (;;) {
-      const int64_t nxt = win + gridDim.x;
+      const int64_t nxt = a.spread ? a.nwin : win + gridDim.x;
       int32_t row2 = -1, c0 = 0, W2 = 0;
       if (nxt < a.nwin) {
         const int64_t s2 = slice_of(nxt, k + 1);
@@ -797,7 +856,7 @@ pcg_batched_persistent(BatchArgs a) {
       X[e] = make_float4(0.f, 0.f, 0.f, 0.f);
       Pv[e] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (!breduce(v, a, parity, S, shw, err)) return;
+    if (!breduce(v, a, parity, S, shw, sh4, err, target)) return;
   }
   if (threadIdx.x < BS) S.bnorm2[threadIdx.x] = S.red[threadIdx.x];
   __syncthreads();
@@ -818,7 +877,7 @@ pcg_batched_persistent(BatchArgs a) {
       }
       R[(int64_t)row * TPR + q] = rf;
     });
-    if (!breduce(v, a, parity, S, shw, err)) return;
+    if (!breduce(v, a, parity, S, shw, sh4, err, target)) return;
   }
   if (threadIdx.x < BS) {
     const int i = threadIdx.x;
@@ -854,7 +913,7 @@ pcg_batched_persistent(BatchArgs a) {
         });
       }
     }
-    if (!bgrid_sync(a.bar, err)) return false;
+    if (!bgrid_sync(a.bar, err, target)) return false;
     if (timed) mark(2);
     Acc2 acc[kIPT];
     if (phase_on(flags)) {
@@ -883,7 +942,7 @@ pcg_batched_persistent(BatchArgs a) {
     double v[kIPT];
 #pragma unroll
     for (int j = 0; j < kIPT; ++j) v[j] = acc[j].get();
-    if (!breduce(v, a, parity, S, shw, err)) return false;
+    if (!breduce(v, a, parity, S, shw, sh4, err, target)) return false;
     if (timed) mark(3);
     return true;
   };
@@ -907,7 +966,7 @@ pcg_batched_persistent(BatchArgs a) {
                             fmaf(bt.z, pv.z, zv.z), fmaf(bt.w, pv.w, zv.w));
       }
     }
-    if (!bgrid_sync(a.bar, err)) return;
+    if (!bgrid_sync(a.bar, err, target)) return;
     mark(-1);
 
     // ---- FP32 iterations until every working instance is frozen
@@ -944,7 +1003,7 @@ pcg_batched_persistent(BatchArgs a) {
         double v[kIPT];
 #pragma unroll
         for (int j = 0; j < kIPT; ++j) v[j] = acc[j].get();
-        if (!breduce(v, a, parity, S, shw, err)) return;
+        if (!breduce(v, a, parity, S, shw, sh4, err, target)) return;
         mark(0);
       }
       if (threadIdx.x < BS) {
@@ -975,7 +1034,7 @@ pcg_batched_persistent(BatchArgs a) {
         double v[kIPT];
 #pragma unroll
         for (int j = 0; j < kIPT; ++j) v[j] = acc[j].get();
-        if (!breduce(v, a, parity, S, shw, err)) return;
+        if (!breduce(v, a, parity, S, shw, sh4, err, target)) return;
         mark(1);
       }
       if (threadIdx.x < BS) {
@@ -987,12 +1046,7 @@ pcg_batched_persistent(BatchArgs a) {
         }
       }
       __syncthreads();   // instances 32..63 are updated by warp 1: count after both
-      if (threadIdx.x == 0) {
-        int c = 0;
-        for (int i = 0; i < BS; ++i) c += S.iterating[i];
-        S.count = c;
-      }
-      __syncthreads();
+      count_flags(S.iterating);
       if (S.count == 0) break;
       // preconditioner on the iterating instances
       if (!apply_precond(S.iterating, true)) return;
@@ -1019,7 +1073,7 @@ pcg_batched_persistent(BatchArgs a) {
           Pv[e] = pv;
         }
       }
-      if (!bgrid_sync(a.bar, err)) return;
+      if (!bgrid_sync(a.bar, err, target)) return;
       mark(4);
       if (timer) ph[5] += 1.0;
     }
@@ -1033,7 +1087,7 @@ pcg_batched_persistent(BatchArgs a) {
         for (int j = 0; j < kIPT; ++j) a.x64[e * kIPT + j] += (double)get4(xv, j);
         X[e] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
-    if (!bgrid_sync(a.bar, err)) return;
+    if (!bgrid_sync(a.bar, err, target)) return;
     {
       double v[kIPT] = {0.0, 0.0, 0.0, 0.0};
       if (any4(S.active))
@@ -1052,7 +1106,7 @@ pcg_batched_persistent(BatchArgs a) {
           }
           R[(int64_t)row * TPR + q] = rf;
         });
-      if (!breduce(v, a, parity, S, shw, err)) return;
+      if (!breduce(v, a, parity, S, shw, sh4, err, target)) return;
     }
     if (threadIdx.x < BS) {
       const int i = threadIdx.x;
@@ -1070,12 +1124,7 @@ pcg_batched_persistent(BatchArgs a) {
       }
     }
     __syncthreads();   // as above: every instance updated before the count
-    if (threadIdx.x == 0) {
-      int c = 0;
-      for (int i = 0; i < BS; ++i) c += S.active[i];
-      S.count = c;
-    }
-    __syncthreads();
+    count_flags(S.active);
     if (S.count == 0) break;
   }
   if (blockIdx.x == 0 && threadIdx.x < BS) {
@@ -1111,8 +1160,10 @@ struct EntryWeights {
 // Per-instance FSAI factors for the batched solve (same definition as the
 // single-instance factor: row i solves L_b[P_i, P_i] g = e_i and stores
 // g / sqrt(g_i)), computed in FP32 from the edge form of L_b and stored in
-// BF16 in CSR order with the instances contiguous: entries with col <= row
-// hold G[row][col], entries with col > row G[col][row].  A group of BS
+// BF16 in the slots of the two halves (pos_lo, pos_hi: slot of a CSR entry
+// of G and G^T), instances contiguous.  The diagonals come from
+// batch_edge_diag_kernel, so that only lower entries are read here (with the
+// rows read whole: 7.0 ms for 16 fields on the 64^3 cube).  A group of BS
 // threads handles one row, thread b instance b, each with the packed lower
 // triangle of its block in shared memory (k <= kBFsaiMax).  Longer rows
 // (about 3 % of the rows at a limit of 12, which lets two blocks share an
@@ -1127,12 +1178,36 @@ constexpr int kBPacked = kBFsaiMax * (kBFsaiMax + 1) / 2;
 
 __device__ __forceinline__ int btri(int r, int c) { return r * (r + 1) / 2 + c; }
 
+// FP32 diagonal of L_b in edge form, [n][BS]: the sum of a free row's weights
+// in CSR order (1 where all are 0)
+__global__ void batch_edge_diag_kernel(int64_t n, int lgB, int B, EntryWeights wt,
+                                       const int32_t* __restrict__ rowptr,
+                                       float* __restrict__ diag) {
+  const int64_t total = n << lgB;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = t >> lgB;
+    const int b = (int)(t & ((1 << lgB) - 1)), inst = b < B ? b : 0;
+    float dsum = 0.0f;
+    for (int32_t k = rowptr[i]; k < rowptr[i + 1]; ++k) dsum += (float)wt(k, inst);
+    diag[t] = dsum == 0.0f ? 1.0f : dsum;
+  }
+}
+
 __global__ void __launch_bounds__(kBFsaiTpb)
 batch_fsai_kernel(int64_t n, int BS, int B, EntryWeights wt, const int32_t* __restrict__ rowptr,
                   const int32_t* __restrict__ col, const int32_t* __restrict__ dpos,
                   const int32_t* __restrict__ pos_up, const uint8_t* __restrict__ tag,
-                  const double* __restrict__ g0, __nv_bfloat16* __restrict__ gb) {
+                  const float* __restrict__ diag, const double* __restrict__ g0,
+                  const int32_t* __restrict__ pos_lo, const int32_t* __restrict__ pos_hi,
+                  __nv_bfloat16* __restrict__ glo, __nv_bfloat16* __restrict__ ghi) {
   extern __shared__ float bsm[];
+  // entry kk of a row's lower half (kk <= its diagonal kd): its slot in G and
+  // that of the transposed entry in G^T
+  auto store = [&](int32_t kk, int32_t kd, int b, __nv_bfloat16 g) {
+    glo[(int64_t)pos_lo[kk] * BS + b] = g;
+    ghi[(int64_t)pos_hi[kk < kd ? pos_up[wt.eid[kk]] : kk] * BS + b] = g;
+  };
   float* A = bsm + threadIdx.x;                                  // stride kBFsaiTpb
   int32_t* P = reinterpret_cast<int32_t*>(bsm + kBPacked * kBFsaiTpb) + threadIdx.x;
   const int stride = kBFsaiTpb;
@@ -1144,11 +1219,7 @@ batch_fsai_kernel(int64_t n, int BS, int B, EntryWeights wt, const int32_t* __re
     const int32_t k0 = rowptr[i], kd = dpos[i];
     const int k = kd - k0 + 1;
     if (k > kBFsaiMax) {   // this row's lower part and its transposed slots
-      for (int32_t kk = k0; kk <= kd; ++kk) {
-        const __nv_bfloat16 g = __float2bfloat16_rn((float)g0[kk]);
-        gb[(int64_t)kk * BS + b] = g;
-        if (kk < kd) gb[(int64_t)pos_up[wt.eid[kk]] * BS + b] = g;
-      }
+      for (int32_t kk = k0; kk <= kd; ++kk) store(kk, kd, b, __float2bfloat16_rn((float)g0[kk]));
       continue;
     }
     for (int qq = 0; qq < k; ++qq) P[qq * stride] = col[k0 + qq];
@@ -1166,19 +1237,17 @@ batch_fsai_kernel(int64_t n, int BS, int B, EntryWeights wt, const int32_t* __re
           if (pass == 0) dmax = fmaxf(dmax, 1.0f);
           continue;
         }
-        float dsum = 0.0f;
+        // lower part of row rw (columns < rw, sorted) merged with P
         int c = 0;
-        for (int32_t kk = rowptr[rw]; kk < rowptr[rw + 1]; ++kk) {
-          const float m = (float)wt(kk, inst);
-          dsum += m;
+        const int32_t kend = dpos[rw];
+        for (int32_t kk = rowptr[rw]; kk < kend; ++kk) {
           const int32_t cc = col[kk];
-          if (kk < dpos[rw]) {            // lower part of row rw: columns < rw
-            while (c < qq && P[c * stride] < cc) ++c;
-            if (c < qq && P[c * stride] == cc && tag[cc] != DEC_NODE_DIRICHLET)
-              A[btri(qq, c) * stride] = -m;
-          }
+          while (c < qq && P[c * stride] < cc) ++c;
+          if (c == qq) break;
+          if (P[c * stride] == cc && tag[cc] != DEC_NODE_DIRICHLET)
+            A[btri(qq, c) * stride] = -(float)wt(kk, inst);
         }
-        A[btri(qq, qq) * stride] = (dsum == 0.0f ? 1.0f : dsum) + shift;
+        A[btri(qq, qq) * stride] = diag[(int64_t)rw * BS + b] + shift;
         if (pass == 0) dmax = fmaxf(dmax, A[btri(qq, qq) * stride]);
       }
       // Cholesky in place; a pivot <= 1e-6 max(diag) marks a singular block
@@ -1206,8 +1275,7 @@ batch_fsai_kernel(int64_t n, int BS, int B, EntryWeights wt, const int32_t* __re
     for (int qq = 0; qq < k; ++qq) {
       const __nv_bfloat16 gq = ok ? __float2bfloat16_rn(A[btri(qq, qq) * stride])
                                   : __float2bfloat16_rn((float)g0[k0 + qq]);
-      gb[(int64_t)(k0 + qq) * BS + b] = gq;
-      if (qq < k - 1) gb[(int64_t)pos_up[wt.eid[k0 + qq]] * BS + b] = gq;
+      store(k0 + qq, kd, b, gq);
     }
   }
 }
@@ -1308,10 +1376,9 @@ __global__ void bbox_fold_kernel(int nb, const double* __restrict__ part, double
 }
 
 // Values of the batched L in its sliced layout, from CSR entry k.
-__global__ void batch_l_values_kernel(int64_t nnz, int kind, int BS, int B,
-                                      const int32_t* __restrict__ pos, EntryWeights wt,
-                                      const double* __restrict__ val64, int2* __restrict__ cw,
-                                      uint8_t* __restrict__ lfc, float* __restrict__ lw,
+__global__ void batch_l_values_kernel(int64_t nnz, int kind, const int32_t* __restrict__ pos,
+                                      EntryWeights wt, const double* __restrict__ val64,
+                                      int2* __restrict__ cw, uint8_t* __restrict__ lfc,
                                       double* __restrict__ l64) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nnz;
        k += (int64_t)gridDim.x * blockDim.x) {
@@ -1320,18 +1387,30 @@ __global__ void batch_l_values_kernel(int64_t nnz, int kind, int BS, int B,
     if (kind == kSets) {
       cw[p].y = __float_as_int((float)val64[k]);
       l64[p] = val64[k];
-    } else if (kind == kStates) {
+    } else {
       const int32_t e = wt.eid[k];
       cw[p].y = __float_as_int((float)wt.w[e]);
       l64[p] = wt.w[e];
       lfc[p] = wt.fc[e];
-    } else {
-      for (int b = 0; b < BS; ++b) {
-        const double we = b < B ? wt(k, b) : 0.0;
-        lw[(int64_t)p * BS + b] = (float)we;
-        l64[(int64_t)p * BS + b] = we;
-      }
     }
+  }
+}
+
+// the same for fields, a thread per entry and instance (a thread per entry
+// wrote its BS values one by one: 1.5 ms for 16 fields on the 64^3 cube)
+__global__ void batch_l_fields_kernel(int64_t nnz, int lgB, int B,
+                                      const int32_t* __restrict__ pos, EntryWeights wt,
+                                      float* __restrict__ lw, double* __restrict__ l64) {
+  const int64_t total = nnz << lgB;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t k = (int32_t)(t >> lgB);
+    const int b = (int)(t & ((1 << lgB) - 1));
+    const int32_t p = pos[k];
+    if (p < 0) continue;
+    const double we = b < B ? wt(k, b) : 0.0;
+    lw[((int64_t)p << lgB) + b] = (float)we;
+    l64[((int64_t)p << lgB) + b] = we;
   }
 }
 
@@ -1367,23 +1446,6 @@ __global__ void batch_g_values_kernel(int64_t nnz, const int32_t* __restrict__ p
     const __nv_bfloat16 g = __float2bfloat16_rn((float)g64[k]);
     if (pos_lo[k] >= 0) glo[pos_lo[k]] = g;
     if (pos_hi[k] >= 0) ghi[pos_hi[k]] = g;
-  }
-}
-
-// per-instance factor halves from the CSR-order per-instance factor
-__global__ void batch_gb_scatter_kernel(int64_t nnz, int BS, const int32_t* __restrict__ pos_lo,
-                                        const int32_t* __restrict__ pos_hi,
-                                        const __nv_bfloat16* __restrict__ gb,
-                                        __nv_bfloat16* __restrict__ glo,
-                                        __nv_bfloat16* __restrict__ ghi) {
-  const int64_t total = nnz * BS;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t k = t / BS;
-    const int b = (int)(t % BS);
-    const __nv_bfloat16 g = gb[t];
-    if (pos_lo[k] >= 0) glo[(int64_t)pos_lo[k] * BS + b] = g;
-    if (pos_hi[k] >= 0) ghi[(int64_t)pos_hi[k] * BS + b] = g;
   }
 }
 
@@ -1459,6 +1521,7 @@ static unsigned grid_for_work(const dec_ctx* ctx, int64_t work) {
 #endif
 constexpr int kTileNodes = DEC_TILE_NODES;
 static dec_status build_morton(dec_ctx* ctx) {
+  if (ctx->order_built) return DEC_OK;   // the order belongs to the mesh
   const int64_t n = ctx->n;
   cudaStream_t s = ctx->stream;
   const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, ctx->num_sms * 4));
@@ -1494,6 +1557,7 @@ static dec_status build_morton(dec_ctx* ctx) {
   invert_order_kernel<<<grid_for_work(ctx, n), 256, 0, s>>>(n, ctx->morton.p, ctx->mrank.p);
   DEC_TRY(cudaGetLastError());
   ctx->launches += 1;
+  ctx->order_built = true;
   return DEC_OK;
 }
 
@@ -1505,12 +1569,16 @@ static dec_status batch_values(dec_ctx* ctx) {
   const int kind = ctx->batch_kind;
   const EntryWeights wt{ctx->eid.p, ctx->w.p, ctx->first_cut.p, ctx->ne, kind};
   const int64_t tL = ctx->bL.total, tlo = ctx->bGlo.total, tup = ctx->bGup.total;
+  int lgB = 3;
+  while ((1 << lgB) < BS) ++lgB;
   // L values
   if (kind == kFields) {
     DEC_TRY(ctx->bLw.ensure((size_t)tL * BS));
     DEC_TRY(ctx->bL64.ensure((size_t)tL * BS));
     DEC_TRY(cudaMemsetAsync(ctx->bLw.p, 0, sizeof(float) * tL * BS, s));
     DEC_TRY(cudaMemsetAsync(ctx->bL64.p, 0, sizeof(double) * tL * BS, s));
+    batch_l_fields_kernel<<<grid_for_work(ctx, nnz * BS), 256, 0, s>>>(
+        nnz, lgB, B, ctx->bL.pos.p, wt, ctx->bLw.p, ctx->bL64.p);
   } else {
     DEC_TRY(ctx->bLcw.ensure(tL));
     DEC_TRY(ctx->bL64.ensure(tL));
@@ -1522,9 +1590,9 @@ static dec_status batch_values(dec_ctx* ctx) {
       DEC_TRY(cudaMemsetAsync(ctx->bLfc.p, 0, tL, s));
     }
   }
-  batch_l_values_kernel<<<grid_for_work(ctx, nnz), 256, 0, s>>>(
-      nnz, kind, BS, B, ctx->bL.pos.p, wt, ctx->val64.p, ctx->bLcw.p, ctx->bLfc.p, ctx->bLw.p,
-      ctx->bL64.p);
+  if (kind != kFields)
+    batch_l_values_kernel<<<grid_for_work(ctx, nnz), 256, 0, s>>>(
+        nnz, kind, ctx->bL.pos.p, wt, ctx->val64.p, ctx->bLcw.p, ctx->bLfc.p, ctx->bL64.p);
   ctx->launches += 1;
   if (kind == kSets) {
     DEC_TRY(ctx->bd32.ensure(n));
@@ -1532,15 +1600,15 @@ static dec_status batch_values(dec_ctx* ctx) {
     batch_diag_kernel<<<grid_for_work(ctx, n), 256, 0, s>>>(n, ctx->dpos.p, ctx->mrank.p,
                                                             ctx->val64.p, ctx->bd32.p,
                                                             ctx->bd64.p);
-    ctx->launches += 1;
+    // shared factor halves
+    DEC_TRY(ctx->bGlo16.ensure(tlo));
+    DEC_TRY(ctx->bGup16.ensure(tup));
+    DEC_TRY(cudaMemsetAsync(ctx->bGlo16.p, 0, sizeof(__nv_bfloat16) * tlo, s));
+    DEC_TRY(cudaMemsetAsync(ctx->bGup16.p, 0, sizeof(__nv_bfloat16) * tup, s));
+    batch_g_values_kernel<<<grid_for_work(ctx, nnz), 256, 0, s>>>(
+        nnz, ctx->bGlo.pos.p, ctx->bGup.pos.p, ctx->g64.p, ctx->bGlo16.p, ctx->bGup16.p);
+    ctx->launches += 2;
   }
-  // shared factor halves
-  DEC_TRY(ctx->bGlo16.ensure(tlo));
-  DEC_TRY(ctx->bGup16.ensure(tup));
-  DEC_TRY(cudaMemsetAsync(ctx->bGlo16.p, 0, sizeof(__nv_bfloat16) * tlo, s));
-  DEC_TRY(cudaMemsetAsync(ctx->bGup16.p, 0, sizeof(__nv_bfloat16) * tup, s));
-  batch_g_values_kernel<<<grid_for_work(ctx, nnz), 256, 0, s>>>(
-      nnz, ctx->bGlo.pos.p, ctx->bGup.pos.p, ctx->g64.p, ctx->bGlo16.p, ctx->bGup16.p);
   // right-hand sides
   DEC_TRY(ctx->bb.ensure((size_t)n * BS));
   batch_rhs_kernel<<<grid_for_work(ctx, n * BS), 256, 0, s>>>(
@@ -1549,10 +1617,12 @@ static dec_status batch_values(dec_ctx* ctx) {
   batch_rhs_unpack_kernel<<<grid_for_work(ctx, n * B), 256, 0, s>>>(n, B, BS, ctx->mrank.p,
                                                                    ctx->bb.p, ctx->b.p);
   DEC_TRY(cudaGetLastError());
-  ctx->launches += 3;
+  ctx->launches += 2;
   if (kind != kSets) {
     // crack states and fields change L per instance: one FSAI factor each
-    DEC_TRY(ctx->bgb.ensure((size_t)nnz * BS));
+    DEC_TRY(ctx->bdiag.ensure((size_t)n * BS));
+    batch_edge_diag_kernel<<<grid_for_work(ctx, n * BS), 256, 0, s>>>(n, lgB, B, wt, ctx->rowptr.p,
+                                                                      ctx->bdiag.p);
     const size_t smem = (size_t)kBPacked * kBFsaiTpb * sizeof(float) +
                         (size_t)kBFsaiMax * kBFsaiTpb * sizeof(int32_t);
     DEC_TRY(cudaFuncSetAttribute(batch_fsai_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1560,15 +1630,14 @@ static dec_status batch_values(dec_ctx* ctx) {
     const int rpb = kBFsaiTpb / BS;
     const unsigned gf = (unsigned)std::max<int64_t>(
         1, std::min<int64_t>((n + rpb - 1) / rpb, (int64_t)ctx->num_sms * 8));
-    batch_fsai_kernel<<<gf, kBFsaiTpb, smem, s>>>(n, BS, B, wt, ctx->rowptr.p, ctx->col.p,
-                                                  ctx->dpos.p, ctx->pos_up.p, ctx->tag.p,
-                                                  ctx->g64.p, ctx->bgb.p);
     DEC_TRY(ctx->bGloB.ensure((size_t)tlo * BS));
     DEC_TRY(ctx->bGupB.ensure((size_t)tup * BS));
     DEC_TRY(cudaMemsetAsync(ctx->bGloB.p, 0, sizeof(__nv_bfloat16) * tlo * BS, s));
     DEC_TRY(cudaMemsetAsync(ctx->bGupB.p, 0, sizeof(__nv_bfloat16) * tup * BS, s));
-    batch_gb_scatter_kernel<<<grid_for_work(ctx, nnz * BS), 256, 0, s>>>(
-        nnz, BS, ctx->bGlo.pos.p, ctx->bGup.pos.p, ctx->bgb.p, ctx->bGloB.p, ctx->bGupB.p);
+    batch_fsai_kernel<<<gf, kBFsaiTpb, smem, s>>>(n, BS, B, wt, ctx->rowptr.p, ctx->col.p,
+                                                  ctx->dpos.p, ctx->pos_up.p, ctx->tag.p,
+                                                  ctx->bdiag.p, ctx->g64.p, ctx->bGlo.pos.p,
+                                                  ctx->bGup.pos.p, ctx->bGloB.p, ctx->bGupB.p);
     DEC_TRY(cudaGetLastError());
     ctx->launches += 2;
     ctx->batch_per_instance = true;
@@ -1587,17 +1656,24 @@ dec_status batch_setup(dec_ctx* ctx) {
   ctx->batch_kind = kind;
   ctx->batch_BS = 0;
   DEC_TRY_STATUS(build_morton(ctx));
-  DEC_TRY_STATUS(build_sell(ctx, kind == kSets ? 4 : 3, ctx->bL, C, R, ctx->morton.p));
-  DEC_TRY_STATUS(build_sell(ctx, 1, ctx->bGlo, C, R, ctx->morton.p));
-  DEC_TRY_STATUS(build_sell(ctx, 2, ctx->bGup, C, R, ctx->morton.p));
-  // rows and columns in Morton positions
-  for (SellLayout* L : {&ctx->bL, &ctx->bGlo, &ctx->bGup}) {
-    const int64_t slots = L->nslices * L->C;
-    renumber_layout_kernel<<<grid_for_work(ctx, std::max<int64_t>(slots, L->total)), 256, 0,
-                             ctx->stream>>>(slots, L->total, ctx->mrank.p, L->perm.p, L->col.p);
-    ctx->launches += 1;
+  // the layouts depend on the mesh, the form of L and the stride only
+  const int form = kind == kSets ? 4 : 3;
+  if (ctx->batch_form != form || ctx->batch_form_BS != BS) {
+    ctx->batch_form = -1;
+    DEC_TRY_STATUS(build_sell(ctx, form, ctx->bL, C, R, ctx->morton.p));
+    DEC_TRY_STATUS(build_sell(ctx, 1, ctx->bGlo, C, R, ctx->morton.p));
+    DEC_TRY_STATUS(build_sell(ctx, 2, ctx->bGup, C, R, ctx->morton.p));
+    // rows and columns in Morton positions
+    for (SellLayout* L : {&ctx->bL, &ctx->bGlo, &ctx->bGup}) {
+      const int64_t slots = L->nslices * L->C;
+      renumber_layout_kernel<<<grid_for_work(ctx, std::max<int64_t>(slots, L->total)), 256, 0,
+                               ctx->stream>>>(slots, L->total, ctx->mrank.p, L->perm.p, L->col.p);
+      ctx->launches += 1;
+    }
+    DEC_TRY(cudaGetLastError());
+    ctx->batch_form = form;
+    ctx->batch_form_BS = BS;
   }
-  DEC_TRY(cudaGetLastError());
   DEC_TRY_STATUS(batch_values(ctx));
   ctx->batch_BS = BS;
   return DEC_OK;
@@ -1751,6 +1827,7 @@ dec_status solve_batched(dec_ctx* ctx, double rtol, int max_iter, int* iters,
   a.rtol2 = rtol * rtol;
   a.seg2 = 1e-4;
   a.max_iter = max_iter;
+  a.spread = a.nwin < grid ? 1 : 0;
   void* args[] = {&a};
   auto launch = [&](int v, int iters_cap) -> cudaError_t {
     a.max_iter = iters_cap;

@@ -161,6 +161,8 @@ struct dec_ctx {
   // [n][BS] vectors
   int batch_kind = 0;                      // 0 Dirichlet sets, 1 crack states, 2 fields
   int batch_BS = 0;                        // instance stride of the layouts
+  bool order_built = false;                // morton, mrank belong to the mesh
+  int batch_form = -1, batch_form_BS = 0;  // what the batched layouts were built for
   dec::DevBuf<int32_t> morton;             // [n] node order of the windows
   dec::DevBuf<int32_t> mrank;              // [n] position of each node in that order
   dec::SellLayout bL, bGlo, bGup;          // L (edge or CSR form), G, G^T
@@ -169,10 +171,10 @@ struct dec_ctx {
   dec::DevBuf<float> bLw;                  // [total][BS] *1 per instance (fields)
   dec::DevBuf<double> bL64;                // FP64 values, [total] or [total][BS]
   dec::DevBuf<float> bd32;                 // [n] diagonal (Dirichlet sets)
+  dec::DevBuf<float> bdiag;                // [n][BS] edge-form diagonals (states, fields)
   dec::DevBuf<double> bd64;
   dec::DevBuf<__nv_bfloat16> bGlo16, bGup16;   // shared factor halves
   dec::DevBuf<__nv_bfloat16> bGloB, bGupB;     // per-instance halves [total][BS]
-  dec::DevBuf<__nv_bfloat16> bgb;          // per-instance factors, CSR order [nnz][BS]
   dec::DevBuf<double> bb, bx64, br64, bpartial;
   dec::DevBuf<int64_t> crack_buf;          // crack growth: block bests, picked edge
   int batch_variant[4] = {0, 0, 0, 0};     // tuned variant + 1 per stride 8..64
@@ -222,9 +224,10 @@ struct dec_ctx {
     sellL.release(); sellLo.release(); sellUp.release(); sL64.release();
     sGlo64.release(); sGup64.release(); sL32.release(); sGlo16.release();
     sGup16.release(); big_rows.release(); coop.release();
+    bdiag.release();
     morton.release(); mrank.release(); bL.release(); bGlo.release(); bGup.release(); bLcw.release();
     bLfc.release(); bLw.release(); bL64.release(); bd32.release(); bd64.release();
-    bGlo16.release(); bGup16.release(); bGloB.release(); bGupB.release(); bgb.release();
+    bGlo16.release(); bGup16.release(); bGloB.release(); bGupB.release();
     bb.release(); bx64.release(); br64.release(); bpartial.release();
     kpartial.release(); crack_buf.release(); bx.release(); br.release(); bz.release();
     bp.release(); bq.release(); bt.release();
