@@ -134,10 +134,16 @@ dec_status dec_mesh_upload(dec_ctx* ctx, const double* xyz, int64_t n_nodes,
   DEC_TRY(upload(ctx->xyz, xyz, 3 * n_nodes, s));
   DEC_TRY(upload(ctx->tets, tets, 4 * n_tets, s));
   DEC_TRY(upload(ctx->tag, node_tag, n_nodes, s));
-  DEC_TRY_STATUS(dec::validate_mesh(ctx));
-  DEC_TRY_STATUS(dec::build_edges(ctx));
-  DEC_TRY_STATUS(dec::build_csr_structure(ctx));
-  DEC_TRY_STATUS(dec::build_sell_layouts(ctx));
+  bool radix = false;
+  int flags = 0;
+  DEC_TRY_STATUS(dec::build_mesh(ctx, &radix));
+  if (!radix) DEC_TRY_STATUS(dec::build_sell_layouts(ctx, &flags));
+  if (radix || (flags & 64)) {     // a node with thousands of edges
+    DEC_TRY(cudaMemsetAsync(ctx->errflag.p, 0, sizeof(int), s));
+    DEC_TRY_STATUS(dec::build_edges(ctx));
+    DEC_TRY_STATUS(dec::build_csr_structure(ctx));
+    DEC_TRY_STATUS(dec::build_sell_layouts(ctx, &flags));
+  }
   ctx->grid_vec = (int)std::max<int64_t>(
       1, std::min<int64_t>((n_nodes + dec::kBlock - 1) / dec::kBlock, (int64_t)ctx->num_sms * 2));
   ctx->grid_sell = (int)std::max<int64_t>(

@@ -389,10 +389,10 @@ dec_status radix_sort_pairs(dec_ctx* ctx, uint64_t* keys, uint32_t* vals,
                             uint64_t* keys_alt, uint32_t* vals_alt, int64_t n,
                             int key_bits, bool* result_in_alt);
 // mesh
-dec_status validate_mesh(dec_ctx* ctx);
+dec_status build_mesh(dec_ctx* ctx, bool* radix);
 dec_status build_edges(dec_ctx* ctx);
 dec_status build_csr_structure(dec_ctx* ctx);
-dec_status build_sell_layouts(dec_ctx* ctx);
+dec_status build_sell_layouts(dec_ctx* ctx, int* flags);
 dec_status build_sell(dec_ctx* ctx, int kind, SellLayout& L, int C, int R,
                       const int32_t* order);
 template <typename T>

@@ -159,10 +159,127 @@ dec_status build_sell(dec_ctx* ctx, int kind, SellLayout& L, int C, int R,
   return DEC_OK;
 }
 
-dec_status build_sell_layouts(dec_ctx* ctx) {
-  DEC_TRY_STATUS(build_sell(ctx, 0, ctx->sellL, 32, kWindow, nullptr));
-  DEC_TRY_STATUS(build_sell(ctx, 1, ctx->sellLo, 32, kWindow, nullptr));
-  DEC_TRY_STATUS(build_sell(ctx, 2, ctx->sellUp, 32, kWindow, nullptr));
+// ---- L, G and G^T in natural order, all three per launch (blockIdx.y)
+struct Sell3 {
+  int32_t* perm[3];
+  int32_t* sptr[3];
+  int32_t* col[3];
+  int32_t* pos[3];
+};
+
+// Rank the rows of each window by (length desc, position asc); `size` gets
+// the entries of every slice (32 times its first row), matrix after matrix
+// with a 0 after each.
+__global__ void __launch_bounds__(kWindow)
+sell3_sort_kernel(int64_t n, int64_t nslices, const int32_t* __restrict__ rowptr,
+                  const int32_t* __restrict__ dpos, Sell3 L, uint32_t* __restrict__ size) {
+  __shared__ __align__(16) int32_t key[kWindow];
+  const int k = blockIdx.y, at = threadIdx.x;
+  const int64_t i = (int64_t)blockIdx.x * kWindow + at;
+  int32_t l = -1;
+  if (i < n) {
+    const int32_t k0 = rowptr[i], k1 = rowptr[i + 1], kd = dpos[i];
+    l = k == 0 ? k1 - k0 : k == 1 ? kd - k0 + 1 : k1 - kd;
+  }
+  key[at] = l;
+  __syncthreads();
+  int rank = 0;
+  const int4* k4 = reinterpret_cast<const int4*>(key);
+#pragma unroll 4
+  for (int j = 0; j < kWindow; j += 4) {
+    const int4 v = k4[j >> 2];
+    rank += (v.x > l || (v.x == l && j < at)) + (v.y > l || (v.y == l && j + 1 < at)) +
+            (v.z > l || (v.z == l && j + 2 < at)) + (v.w > l || (v.w == l && j + 3 < at));
+  }
+  L.perm[k][(int64_t)blockIdx.x * kWindow + rank] = i < n ? (int32_t)i : -1;
+  const int64_t s = (int64_t)blockIdx.x * (kWindow / 32) + rank / 32;
+  if (rank % 32 == 0) size[k * (nslices + 1) + s] = 32u * (uint32_t)(l < 0 ? 0 : l);
+  if (s == nslices - 1 && rank % 32 == 0) size[k * (nslices + 1) + nslices] = 0u;
+}
+
+// slice pointers of each matrix from the scan over all three
+__global__ void sell3_sptr_kernel(int64_t nslices, const uint32_t* __restrict__ scan, Sell3 L) {
+  const int k = blockIdx.y;
+  const uint32_t* a = scan + k * (nslices + 1);
+  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s <= nslices;
+       s += (int64_t)gridDim.x * blockDim.x)
+    L.sptr[k][s] = (int32_t)(a[s] - a[0]);
+}
+
+__global__ void sell3_fill_kernel(int64_t nslices, const int32_t* __restrict__ rowptr,
+                                  const int32_t* __restrict__ dpos,
+                                  const int32_t* __restrict__ csr_col, Sell3 L) {
+  const int k = blockIdx.y;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, s = t >> 5;
+  if (s >= nslices) return;
+  const int32_t r = L.perm[k][t], base = L.sptr[k][s] + (int32_t)(t & 31);
+  const int32_t end = L.sptr[k][s + 1];
+  int32_t p = base;
+  if (r >= 0) {
+    const int32_t k0 = rowptr[r], k1 = rowptr[r + 1], kd = dpos[r];
+    const int32_t b = k == 2 ? kd : k0, e = k == 1 ? kd + 1 : k1;
+    for (int32_t j = k0; j < b; ++j) L.pos[k][j] = -1;
+    for (int32_t j = b; j < e; ++j, p += 32) {
+      L.col[k][p] = csr_col[j];
+      L.pos[k][j] = p;
+    }
+    for (int32_t j = e; j < k1; ++j) L.pos[k][j] = -1;
+  }
+  // padding: value 0, a column already in cache (the row itself)
+  for (; p < end; p += 32) L.col[k][p] = r >= 0 ? r : 0;
+}
+
+// *flags: errflag as the mesh build left it, read with the sizes
+dec_status build_sell_layouts(dec_ctx* ctx, int* flags) {
+  const int64_t n = ctx->n;
+  cudaStream_t s = ctx->stream;
+  SellLayout* M[3] = {&ctx->sellL, &ctx->sellLo, &ctx->sellUp};
+  const int64_t nwin = (n + kWindow - 1) / kWindow, ns = nwin * (kWindow / 32);
+  Sell3 a;
+  for (int k = 0; k < 3; ++k) {
+    M[k]->C = 32;
+    M[k]->R = kWindow;
+    M[k]->nslices = ns;
+    DEC_TRY(M[k]->perm.ensure(nwin * kWindow));
+    DEC_TRY(M[k]->sptr.ensure(ns + 1));
+    DEC_TRY(M[k]->pos.ensure(ctx->nnz));
+    a.perm[k] = M[k]->perm.p;
+    a.sptr[k] = M[k]->sptr.p;
+    a.pos[k] = M[k]->pos.p;
+    a.col[k] = nullptr;
+  }
+  const int64_t cnt = 3 * (ns + 1);
+  DEC_TRY(ctx->flags.ensure(cnt));
+  DEC_TRY(ctx->scan_tmp.ensure(scan_tmp_size(cnt)));
+  sell3_sort_kernel<<<dim3((unsigned)nwin, 3), kWindow, 0, s>>>(n, ns, ctx->rowptr.p, ctx->dpos.p, a,
+                                                                ctx->flags.p);
+  DEC_TRY(cudaGetLastError());
+  DEC_TRY(exclusive_scan_u32(ctx->flags.p, ctx->flags.p, cnt, ctx->scan_tmp.p, ctx->scan_tmp.cap,
+                             s));
+  sell3_sptr_kernel<<<dim3((unsigned)std::min<int64_t>((ns + 256) / 256, 2048), 3), 256, 0, s>>>(
+      ns, ctx->flags.p, a);
+  DEC_TRY(cudaGetLastError());
+  uint32_t end[3];
+  for (int k = 0; k < 3; ++k)
+    DEC_TRY(cudaMemcpyAsync(end + k, ctx->flags.p + k * (ns + 1) + ns, sizeof(uint32_t),
+                            cudaMemcpyDeviceToHost, s));
+  DEC_TRY(cudaMemcpyAsync(flags, ctx->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+  DEC_TRY(cudaStreamSynchronize(s));
+  ctx->launches += 5;
+  if (*flags & 64) return DEC_OK;
+  uint32_t before = 0;
+  for (int k = 0; k < 3; ++k) {
+    M[k]->total = (uint32_t)(end[k] - before);   // a matrix has fewer than 2^32 entries
+    before = end[k];
+    if (M[k]->total >= (int64_t)INT32_MAX)
+      return ctx->fail(DEC_ERR_LIMIT, "sliced layout: more than 2^31 - 1 entries");
+    DEC_TRY(M[k]->col.ensure(M[k]->total));
+    a.col[k] = M[k]->col.p;
+  }
+  sell3_fill_kernel<<<dim3((unsigned)((ns * 32 + 255) / 256), 3), 256, 0, s>>>(
+      ns, ctx->rowptr.p, ctx->dpos.p, ctx->col.p, a);
+  DEC_TRY(cudaGetLastError());
+  ctx->launches += 1;
   return DEC_OK;
 }
 

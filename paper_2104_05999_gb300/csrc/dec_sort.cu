@@ -114,6 +114,10 @@ cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n,
   if (n <= 0) return cudaSuccess;
   int64_t nb = (n + kScanTile - 1) / kScanTile;
   if ((size_t)nb > tmp_cap) return cudaErrorInvalidValue;
+  if (in == out && n <= 8 * 1024) {      // one block, one launch
+    scan_top_kernel<<<1, 1024, 0, s>>>(out, n);
+    return cudaGetLastError();
+  }
   scan_reduce_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(in, tmp, n);
   scan_top_kernel<<<1, 1024, 0, s>>>(tmp, nb);
   scan_down_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, tmp, n);
