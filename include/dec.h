@@ -80,7 +80,9 @@ enum {
 };
 /* solve modes (dec_solve) */
 enum {
-  DEC_MODE_FP64 = 0,   /* PCG in FP64 (matrix, preconditioner, vectors)       */
+  DEC_MODE_FP64 = 0,   /* PCG in FP64 (matrix, preconditioner, vectors): one
+                          launch per instance up to 6,000 nodes, one kernel
+                          per phase above                                  */
   DEC_MODE_MIXED = 1,  /* PCG with FP32 vectors and L and a BF16 FSAI factor
                           (FP32 Jacobi) inside FP64 defect correction: the
                           FP32 update is added to an FP64 solution x and the
@@ -259,9 +261,11 @@ dec_status dec_get_batch_variant(dec_ctx* ctx, int32_t* gather_entries);
  * shape on the context's scratch vectors and keeps the fastest.
  *   precision  0: FP64 (DEC_MODE_FP64), 1: FP32 / BF16 (mixed modes).
  *   l_shape    host: 100 * (resident blocks per SM) + (matrix entries per
- *              round trip): one of 408, 808, 412, 804; 0 before any solve.
+ *              round trip): one of 408, 808, 412, 804; 0 before any solve
+ *              with these kernels (DEC_MODE_FP64 takes them above 6,000 nodes
+ *              or when a shape is forced).
  *   g_shape    host: 14 (slices staged in shared memory) or 8 (round trips
- *              of 8 entries); 0 before any solve with FSAI.
+ *              of 8 entries); 0 before any such solve with FSAI.
  * Every shape gives bit-identical results.  (No counterpart in the paper:
  * a launch-shape choice.) */
 dec_status dec_get_sell_variant(const dec_ctx* ctx, int32_t precision, int32_t* l_shape,

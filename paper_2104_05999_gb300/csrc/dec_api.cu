@@ -257,15 +257,11 @@ dec_status dec_laplacian_build(dec_ctx* ctx, const double* T0, int32_t n_sets,
   const int V = shared ? 1 : std::max(ctx->n_scales, ctx->n_fields);  // value sets
   DEC_TRY(upload(ctx->T0, T0, (int64_t)n_sets * n, s));
   DEC_TRY(ctx->val64.ensure((size_t)V * nnz));
-  DEC_TRY(ctx->sL64.ensure((size_t)V * ctx->sellL.total));
-  DEC_TRY(ctx->sL32.ensure((size_t)V * ctx->sellL.total));
+  // the solver's copies of the values are made by the solves that use them
+  ctx->sell_have.assign(V, 0);
   DEC_TRY(ctx->b.ensure((size_t)ctx->B * n));
   if (precond != DEC_PRECOND_JACOBI) {
     DEC_TRY(ctx->g64.ensure((size_t)V * nnz));
-    DEC_TRY(ctx->sGlo64.ensure((size_t)V * ctx->sellLo.total));
-    DEC_TRY(ctx->sGup64.ensure((size_t)V * ctx->sellUp.total));
-    DEC_TRY(ctx->sGlo16.ensure((size_t)V * ctx->sellLo.total));
-    DEC_TRY(ctx->sGup16.ensure((size_t)V * ctx->sellUp.total));
   } else {
     DEC_TRY(ctx->dinv64.ensure((size_t)V * n));
     DEC_TRY(ctx->dinv32.ensure((size_t)V * n));

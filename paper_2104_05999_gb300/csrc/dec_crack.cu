@@ -210,16 +210,13 @@ dec_status crack_paths(dec_ctx* ctx, int P, int max_steps, const int32_t* orders
   ctx->n_fields = P;
   ctx->B = P;
   ctx->precond = DEC_PRECOND_FSAI_SHARED;
+  ctx->sell_have.assign(1, 0);
   DEC_TRY(ctx->b.ensure((size_t)P * n));
   DEC_TRY(ctx->u.ensure((size_t)P * n));
   DEC_TRY(ctx->out3.ensure(3 * (size_t)P + 2));
   // the shared FSAI factor (kept by long rows) needs its buffers even when
   // the context was built with Jacobi
   DEC_TRY(ctx->g64.ensure(ctx->nnz));
-  DEC_TRY(ctx->sGlo64.ensure(ctx->sellLo.total));
-  DEC_TRY(ctx->sGup64.ensure(ctx->sellUp.total));
-  DEC_TRY(ctx->sGlo16.ensure(ctx->sellLo.total));
-  DEC_TRY(ctx->sGup16.ensure(ctx->sellUp.total));
   DEC_TRY_STATUS(build_values(ctx, 0));
   DEC_TRY_STATUS(build_precond(ctx, 0));   // the factor long rows keep
   DEC_TRY_STATUS(batch_setup(ctx));

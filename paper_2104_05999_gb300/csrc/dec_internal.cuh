@@ -143,6 +143,7 @@ struct dec_ctx {
   dec::DevBuf<double> dinv64;      // [B][n]
   // solver state
   dec::DevBuf<double> x64, r64, z64, p64, q64, t64, u;  // u: [B][n] result
+  dec::DevBuf<double> p64b, r64b;  // second buffers of p and r
   dec::DevBuf<float> x32, r32, z32, p32, q32, t32, r32b, p32b;
   dec::DevBuf<double> partial;     // [kRedSlots][reduce_grid]
   dec::DevBuf<unsigned> ticket;
@@ -155,6 +156,7 @@ struct dec_ctx {
   dec::DevBuf<double> sL64, sGlo64, sGup64;
   dec::DevBuf<float> sL32;
   dec::DevBuf<__nv_bfloat16> sGlo16, sGup16;
+  std::vector<uint8_t> sell_have;  // per value set: SELL copies made (1: FP64, 2: FP32 / BF16)
   dec::DevBuf<int32_t> big_rows;   // FSAI rows for the warp-per-row kernel
   dec::DevBuf<int64_t> coop;       // persistent solve: barrier, status, result
   // batched solve: sliced layouts over spatial windows, per-entry data,
@@ -224,7 +226,7 @@ struct dec_ctx {
     sellL.release(); sellLo.release(); sellUp.release(); sL64.release();
     sGlo64.release(); sGup64.release(); sL32.release(); sGlo16.release();
     sGup16.release(); big_rows.release(); coop.release();
-    bdiag.release();
+    bdiag.release(); p64b.release(); r64b.release();
     morton.release(); mrank.release(); bL.release(); bGlo.release(); bGup.release(); bLcw.release();
     bLfc.release(); bLw.release(); bL64.release(); bd32.release(); bd64.release();
     bGlo16.release(); bGup16.release(); bGloB.release(); bGupB.release();
@@ -414,6 +416,12 @@ dec_status k_eff_all(dec_ctx* ctx, double* out3_host);   // [B][3], one pass
 dec_status form_T(dec_ctx* ctx, int inst, double* T);
 dec_status solve_mixed_persistent(dec_ctx* ctx, int inst, double rtol, int max_iter,
                                   int* iters_out, double* relres_out);
+// FP64 PCG of a small system in one launch of a thread-block cluster
+dec_status solve_fp64_cluster(dec_ctx* ctx, int inst, double rtol, int max_iter, bool warm,
+                              int* iters_out, double* relres_out);
+// SELL copies of value set vs (bits 1: FP64, 2: FP32 and BF16), made on the
+// first use after a build
+dec_status sell_copies(dec_ctx* ctx, int vs, int bits);
 dec_status batch_setup(dec_ctx* ctx);
 // warm: start every instance from the last batched solution
 dec_status solve_batched(dec_ctx* ctx, double rtol, int max_iter, int* iters,

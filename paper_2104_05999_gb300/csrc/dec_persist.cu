@@ -18,6 +18,9 @@
 #include "dec_kern.cuh"
 
 #include <algorithm>
+#include <cooperative_groups.h>
+#include <cmath>
+#include <cstring>
 #include <type_traits>
 
 namespace dec {
@@ -120,20 +123,19 @@ __device__ __forceinline__ bool grid_sum(const T (&v)[NV], double (&tot)[NV],
 // the fly: sum_j a_j * (X[c_j] + coef * Y[c_j]).  Used to fuse the vector
 // update that produced the operand into the product that consumes it (the
 // owner of row c computes the same fmaf for its own entry, so both agree).
-template <typename MT>
-__device__ __forceinline__ float sell_row2(const SellArg<MT>& A, int64_t s, int lane,
-                                           const float* __restrict__ X,
-                                           const float* __restrict__ Y, float coef) {
+template <typename MT, typename VT>
+__device__ __forceinline__ VT sell_row2(const SellArg<MT>& A, int64_t s, int lane, const VT* X,
+                                        const VT* Y, VT coef) {
   constexpr int U = 8;
   const int32_t base = __ldg(A.sptr + s);
   const int32_t w = (__ldg(A.sptr + s + 1) - base) >> 5;
   const int32_t* __restrict__ cp = A.col + base + lane;
   const MT* __restrict__ vp = A.val + base + lane;
-  float acc = 0.0f;
+  VT acc = VT(0);
   for (int32_t j = 0; j < w; j += U) {
     int32_t c[U];
     MT av[U];
-    float xv[U], yv[U];
+    VT xv[U], yv[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const bool ok = j + u < w;
@@ -142,12 +144,12 @@ __device__ __forceinline__ float sell_row2(const SellArg<MT>& A, int64_t s, int 
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      xv[u] = j + u < w ? X[c[u]] : 0.0f;
-      yv[u] = j + u < w ? Y[c[u]] : 0.0f;
+      xv[u] = j + u < w ? X[c[u]] : VT(0);
+      yv[u] = j + u < w ? Y[c[u]] : VT(0);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (j + u < w) acc = fma_(av[u], fmaf(coef, yv[u], xv[u]), acc);
+      if (j + u < w) acc = fma_(av[u], fma_(coef, yv[u], xv[u]), acc);
   }
   return acc;
 }
@@ -384,6 +386,7 @@ dec_status solve_mixed_persistent(dec_ctx* ctx, int inst, double rtol, int max_i
   if (per_sm < 1) return DEC_ERR_LIMIT;
   const int grid = ctx->num_sms;   // one block per SM (per_sm >= 1 checked)
   DEC_TRY(ctx->partial.ensure((size_t)kRedSlots * std::max(grid, ctx->reduce_grid)));
+  DEC_TRY_STATUS(sell_copies(ctx, vs, 2));
   DEC_TRY(ctx->coop.ensure(16));
   unsigned* bar = reinterpret_cast<unsigned*>(ctx->coop.p);
   int* status = reinterpret_cast<int*>(ctx->coop.p + 2);
@@ -425,6 +428,394 @@ dec_status solve_mixed_persistent(dec_ctx* ctx, int inst, double rtol, int max_i
   if (hs[0]) return ctx->fail(DEC_ERR_TIMEOUT, "persistent solve: a grid barrier timed out");
   if (hs[2] == 1) return ctx->fail(DEC_NOT_CONVERGED, "max_iter reached");
   if (hs[2] == 2) return ctx->fail(DEC_NOT_CONVERGED, "residual replacement stalled");
+  return DEC_OK;
+}
+
+// ------------------------------------------- FP64 PCG of small systems
+// One cluster of 16 blocks runs the whole FP64 solve of up to
+// kClusterRows nodes: the three phases per iteration of the kernel above,
+// separated by cluster barriers, block sums exchanged through distributed
+// shared memory.  Bound by latency: a phase is one round of gathers from L2,
+// a sum in the block and a cluster barrier.  Whole solve to 1e-10 at 3,375
+// nodes with FSAI, 47 iterations: 788 us (16.8 us an iteration, set-up and
+// read-back included) against 1,415 us for five kernels per iteration in a
+// graph; at 729 nodes 432 against 905 us.  Eight blocks that read the matrix
+// from L2, two slices a warp, took 988 us.
+constexpr int kCBlock = 512;
+constexpr int kCBlocks = 16;
+
+struct ClusterArgs {
+  int64_t n;
+  SellArg<double> A, Glo, Gup;
+  const double* dinv;         // Jacobi, or nullptr for FSAI
+  const double* b;
+  double* x;                  // start (warm) and solution
+  double *r[2], *p[2], *z, *q, *t;
+  double rtol2;
+  int max_iter, warm;
+  int cap;                    // entries a block's shared memory holds
+  int* status;                // [0] iterations, [1] 0 converged, 1 max_iter, 3 breakdown
+  double* result;             // [0] |b - L x|^2, [1] |b|^2
+};
+
+// store v at block b's copy of the shared address `at`
+__device__ __forceinline__ void store_cluster(uint32_t at, int b, double v) {
+  asm volatile(
+      "{\n\t.reg .b32 remote;\n\t"
+      "mapa.shared::cluster.u32 remote, %0, %1;\n\t"
+      "st.shared::cluster.f64 [remote], %2;\n\t}"
+      :: "r"(at), "r"(b), "d"(v) : "memory");
+}
+
+template <bool JACOBI>
+__global__ void __launch_bounds__(kCBlock, 1)
+pcg_cluster_kernel(ClusterArgs a) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ double sh[2][kCBlock];
+  __shared__ double slot[2][2][kCBlocks][32];   // [parity][value][block][lane]
+  __shared__ double bc[3];                      // sums and a ratio for the whole block
+  const int rank = (int)cluster.block_rank();
+  const int64_t n = a.n;
+  const int64_t gtid = (int64_t)rank * kCBlock + threadIdx.x;
+  const int64_t gstride = (int64_t)kCBlocks * kCBlock;
+  const int lane = threadIdx.x & 31;
+  // consecutive slices on different SMs
+  const int64_t gwarp = (int64_t)(threadIdx.x >> 5) * kCBlocks + rank;
+  int parity = 0;
+  // Sums of one or two values over the cluster, in a fixed order, into
+  // bc[0..1] of every block; also the barrier between phases.  finish(s0, s1)
+  // goes to bc[2].  One FP64 instruction of a warp holds the SM's pipe for 16
+  // cycles, so one warp adds the block's values lane by lane, the 32 lane
+  // sums of each block are exchanged, and only their total takes a butterfly.
+  auto sum2 = [&](double v0, double v1, auto two_c, auto&& finish) {
+    constexpr int NV = decltype(two_c)::value ? 2 : 1;
+    sh[0][threadIdx.x] = v0;
+    if constexpr (NV == 2) sh[1][threadIdx.x] = v1;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        double t[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) t[c] = sh[k][32 * c + lane];
+#pragma unroll
+        for (int w = 4; w < kCBlock / 32; ++w) t[w & 3] += sh[k][32 * w + lane];
+        const double own = (t[0] + t[1]) + (t[2] + t[3]);
+        const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&slot[parity][k][rank][lane]);
+#pragma unroll 4
+        for (int b = 0; b < kCBlocks; ++b) store_cluster(mine, b, own);
+      }
+    }
+    cluster.sync();
+    if (threadIdx.x < 32) {
+      double tot[2] = {0.0, 0.0};
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        double t[2] = {slot[parity][k][0][lane], slot[parity][k][1][lane]};
+#pragma unroll
+        for (int b = 2; b < kCBlocks; ++b) t[b & 1] += slot[parity][k][b][lane];
+        tot[k] = t[0] + t[1];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], o);
+      }
+      if (lane == 0) {
+        bc[0] = tot[0];
+        bc[1] = tot[1];
+        bc[2] = finish(tot[0], tot[1]);
+      }
+    }
+    parity ^= 1;
+    __syncthreads();
+  };
+  using One = std::false_type;
+  using Two = std::true_type;
+  auto nothing = [](double, double) { return 0.0; };
+  // This warp's slice of each matrix.
+  constexpr int kL = 0, kLo = 1, kUp = 2;
+  extern __shared__ __align__(16) double cvals[];
+  uint16_t* ccols = reinterpret_cast<uint16_t*>(cvals + a.cap);
+  __shared__ int used;
+  if (threadIdx.x == 0) used = 0;
+  __syncthreads();
+  int32_t off[3], wid[3], row_of[3];   // first slot + lane, width, this lane's row
+  int32_t entries = 0;
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    const SellArg<double>& A = m == kL ? a.A : m == kLo ? a.Glo : a.Gup;
+    const bool have = (m == kL || !JACOBI) && gwarp < A.nslices;
+    off[m] = have ? __ldg(A.sptr + gwarp) + lane : 0;
+    wid[m] = have ? (__ldg(A.sptr + gwarp + 1) - __ldg(A.sptr + gwarp)) >> 5 : 0;
+    row_of[m] = have ? __ldg(A.perm + 32 * gwarp + lane) : -1;
+    entries += 32 * wid[m];
+  }
+  int32_t at = 0;
+  if (lane == 0) at = atomicAdd(&used, entries);
+  at = __shfl_sync(0xffffffffu, at, 0) + lane;
+  __syncthreads();
+  // Entries in shared memory (16-bit columns) where a block's all fit: of the
+  // three dependent trips to L2 per phase (column, operand, then the sum) the
+  // operand's is left.
+  const bool staged = used <= a.cap;
+  if (staged) {
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const SellArg<double>& A = m == kL ? a.A : m == kLo ? a.Glo : a.Gup;
+      for (int32_t j = 0; j < wid[m]; ++j) {
+        cvals[at + 32 * j] = __ldg(A.val + off[m] + 32 * j);
+        ccols[at + 32 * j] = (uint16_t)__ldg(A.col + off[m] + 32 * j);
+      }
+      off[m] = at;
+      at += 32 * wid[m];
+    }
+    __syncwarp();
+  }
+  auto run = [&](auto staged_c) {
+  constexpr bool STAGED = decltype(staged_c)::value;
+  // For this warp's rows of matrix m: own(row) before the products,
+  // body(row, product, own) after them; the operand is X[c] (TWO: X[c] +
+  // coef Y[c]).  The loads of a round are issued before any is used.
+  auto product = [&](auto two_c, auto m_c, const double* X, const double* Y, double coef,
+                     auto&& own, auto&& body) {
+    constexpr bool TWO = decltype(two_c)::value;
+    constexpr int m = decltype(m_c)::value;
+    constexpr int U = TWO ? 4 : 6;   // more spill registers at 512 threads: 24 ms, not 21.7
+    const SellArg<double>& A = m == kL ? a.A : m == kLo ? a.Glo : a.Gup;
+    const int32_t w = wid[m], row = row_of[m];
+    double2 mine = make_double2(0.0, 0.0);
+    if (row >= 0) mine = own(row);
+    double acc = 0.0;
+#pragma unroll 1
+    for (int32_t j = 0; j < w; j += U) {
+      double xv[U], yv[TWO ? U : 1];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (j + u < w) {
+          const int32_t e = off[m] + 32 * (j + u);
+          const int32_t c = STAGED ? (int32_t)ccols[e] : __ldg(A.col + e);
+          xv[u] = X[c];
+          if constexpr (TWO) yv[u] = Y[c];
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (j + u < w) {
+          const int32_t e = off[m] + 32 * (j + u);
+          const double v = STAGED ? cvals[e] : __ldg(A.val + e);
+          if constexpr (TWO) acc = fma(v, fma(coef, yv[u], xv[u]), acc);
+          else acc = fma(v, xv[u], acc);
+        }
+    }
+    if (row >= 0) body(row, acc, mine);
+  };
+  using L0 = std::integral_constant<int, kL>;
+  using LO = std::integral_constant<int, kLo>;
+  using UP = std::integral_constant<int, kUp>;
+  auto plain = [&](auto m_c, const double* X, auto&& own, auto&& body) {
+    product(std::false_type{}, m_c, X, (const double*)nullptr, 0.0, own, body);
+  };
+  auto fused = [&](auto m_c, const double* X, const double* Y, double coef, auto&& own,
+                   auto&& body) {
+    product(std::true_type{}, m_c, X, Y, coef, own, body);
+  };
+  auto none = [](int32_t) { return make_double2(0.0, 0.0); };
+  int cur = 0, pc = 0;
+  // r = b - L x, r.r in bc[0]
+  auto residual = [&]() {
+    double rr = 0.0;
+    double* r = a.r[cur];
+    plain(L0{}, a.x, [&](int32_t row) { return make_double2(a.b[row], 0.0); },
+          [&](int32_t row, double acc, double2 o) {
+            const double ri = o.x - acc;
+            r[row] = ri;
+            rr = fma(ri, ri, rr);
+          });
+    sum2(rr, 0.0, One{}, nothing);
+  };
+
+  {
+    double bb = 0.0;
+    for (int64_t i = gtid; i < n; i += gstride) {
+      const double bi = a.b[i];
+      if (!a.warm) {
+        a.x[i] = 0.0;
+        a.r[0][i] = bi;
+      }
+      a.p[0][i] = 0.0;
+      bb = fma(bi, bi, bb);
+    }
+    sum2(bb, 0.0, One{}, nothing);
+  }
+  const double bnorm2 = bc[0], tol2 = a.rtol2 * bnorm2;
+  double rr = bnorm2;
+  if (a.warm && bnorm2 > 0.0) {
+    residual();
+    rr = bc[0];
+  }
+  int iters = 0, outcome = 0;
+  while (bnorm2 > 0.0 && !(rr <= tol2)) {
+    // (re)start: z = M r, r.z, beta = 0
+    double v = 0.0;
+    const double* rc = a.r[cur];
+    if (JACOBI) {
+      for (int64_t i = gtid; i < n; i += gstride) {
+        const double zi = a.dinv[i] * rc[i];
+        a.z[i] = zi;
+        v = fma(rc[i], zi, v);
+      }
+    } else {
+      plain(LO{}, rc, none, [&](int32_t row, double acc, double2) { a.t[row] = acc; });
+      cluster.sync();
+      plain(UP{}, a.t, [&](int32_t row) { return make_double2(rc[row], 0.0); },
+            [&](int32_t row, double acc, double2 o) {
+              a.z[row] = acc;
+              v = fma(o.x, acc, v);
+            });
+    }
+    sum2(v, 0.0, One{}, nothing);
+    double rz = bc[0], beta = 0.0;
+    bool breakdown = false;
+    for (;;) {
+      // A: p = z + beta p, q = L p, p.q
+      const double* po = a.p[pc];
+      double* pn = a.p[pc ^ 1];
+      double acc = 0.0;
+      fused(L0{}, a.z, po, beta, [&](int32_t row) { return make_double2(po[row], a.z[row]); },
+            [&](int32_t row, double qi, double2 o) {
+              const double pi = fma(beta, o.x, o.y);
+              pn[row] = pi;
+              a.q[row] = qi;
+              acc = fma(pi, qi, acc);
+            });
+      sum2(acc, 0.0, One{}, [&](double s, double) { return rz / s; });
+      pc ^= 1;
+      const double pq = bc[0], alpha = bc[2];
+      if (!(pq > 0.0) || !isfinite(pq)) { breakdown = true; break; }
+      // B: r' = r - alpha q, x += alpha p, r'.r', t = G r' (Jacobi: z, r'.z)
+      const double* ro = a.r[cur];
+      double* rn = a.r[cur ^ 1];
+      double s0 = 0.0, s1 = 0.0;
+      if constexpr (JACOBI) {
+        for (int64_t i = gtid; i < n; i += gstride) {
+          const double ri = fma(-alpha, a.q[i], ro[i]);
+          rn[i] = ri;
+          a.x[i] = fma(alpha, pn[i], a.x[i]);
+          s0 = fma(ri, ri, s0);
+          const double zi = a.dinv[i] * ri;
+          a.z[i] = zi;
+          s1 = fma(ri, zi, s1);
+        }
+      } else {
+        fused(LO{}, ro, a.q, -alpha,
+              [&](int32_t row) {
+                return make_double2(fma(-alpha, a.q[row], ro[row]),
+                                    fma(alpha, pn[row], a.x[row]));
+              },
+              [&](int32_t row, double ti, double2 o) {
+                rn[row] = o.x;
+                a.x[row] = o.y;
+                a.t[row] = ti;
+                s0 = fma(o.x, o.x, s0);
+              });
+      }
+      sum2(s0, s1, std::bool_constant<JACOBI>{}, [&](double, double s) { return s / rz; });
+      cur ^= 1;
+      ++iters;
+      rr = bc[0];
+      if (rr <= tol2 || iters >= a.max_iter || !isfinite(rr)) break;
+      if constexpr (JACOBI) {
+        rz = bc[1];
+      } else {
+        // C: z = G^T t, r'.z
+        double w = 0.0;
+        plain(UP{}, a.t, [&](int32_t row) { return make_double2(rn[row], 0.0); },
+              [&](int32_t row, double zi, double2 o) {
+                a.z[row] = zi;
+                w = fma(o.x, zi, w);
+              });
+        sum2(w, 0.0, One{}, [&](double s, double) { return s / rz; });
+        rz = bc[0];
+      }
+      beta = bc[2];
+    }
+    // the true residual decides
+    residual();
+    rr = bc[0];
+    if (breakdown) { outcome = 3; break; }
+    if (rr <= tol2) break;
+    if (iters >= a.max_iter) { outcome = 1; break; }
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    a.status[0] = iters;
+    a.status[1] = outcome;
+    a.result[0] = bnorm2 > 0.0 ? rr : 0.0;
+    a.result[1] = bnorm2;
+  }
+  };
+  if (staged) run(std::true_type{});
+  else run(std::false_type{});
+  cluster.sync();     // no block leaves while another may write its slots
+}
+
+dec_status solve_fp64_cluster(dec_ctx* ctx, int inst, double rtol, int max_iter, bool warm,
+                              int* iters_out, double* relres_out) {
+  const int64_t n = ctx->n;
+  const int vs = value_set(ctx, inst);
+  cudaStream_t s = ctx->stream;
+  const bool fsai = ctx->precond == DEC_PRECOND_FSAI;
+  DEC_TRY_STATUS(sell_copies(ctx, vs, 1));
+  DEC_TRY(ctx->coop.ensure(16));
+  DEC_TRY(ctx->p64b.ensure(n));
+  DEC_TRY(ctx->r64b.ensure(n));
+  ClusterArgs a{};
+  a.n = n;
+  a.A = sell_arg(ctx->sellL, ctx->sL64.p + (int64_t)vs * ctx->sellL.total);
+  a.Glo = sell_arg(ctx->sellLo, fsai ? ctx->sGlo64.p + (int64_t)vs * ctx->sellLo.total : nullptr);
+  a.Gup = sell_arg(ctx->sellUp, fsai ? ctx->sGup64.p + (int64_t)vs * ctx->sellUp.total : nullptr);
+  a.dinv = fsai ? nullptr : ctx->dinv64.p + (int64_t)vs * n;
+  a.b = ctx->b.p + (int64_t)inst * n;
+  a.x = ctx->u.p + (int64_t)inst * n;
+  a.r[0] = ctx->r64.p;
+  a.r[1] = ctx->r64b.p;
+  a.p[0] = ctx->p64.p;
+  a.p[1] = ctx->p64b.p;
+  a.z = ctx->z64.p;
+  a.q = ctx->q64.p;
+  a.t = ctx->t64.p;
+  a.rtol2 = rtol * rtol;
+  a.max_iter = max_iter;
+  a.warm = warm ? 1 : 0;
+  a.status = reinterpret_cast<int*>(ctx->coop.p + 2);
+  a.result = reinterpret_cast<double*>(ctx->coop.p + 8);
+  a.cap = 19 * 1024;          // 190 KB of values and 16-bit columns
+  const int smem = a.cap * (int)(sizeof(double) + sizeof(uint16_t));
+  auto kern = fsai ? pcg_cluster_kernel<false> : pcg_cluster_kernel<true>;
+  DEC_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  DEC_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kCBlocks;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kCBlocks);
+  cfg.blockDim = dim3(kCBlock);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  DEC_TRY(cudaLaunchKernelEx(&cfg, kern, a));
+  DEC_TRY(cudaGetLastError());
+  ctx->launches += 1;
+  int64_t h[16];
+  DEC_TRY(cudaMemcpyAsync(h, ctx->coop.p, sizeof(h), cudaMemcpyDeviceToHost, s));
+  DEC_TRY(cudaStreamSynchronize(s));
+  int hs[2];
+  double hr[2];
+  memcpy(hs, h + 2, sizeof(hs));
+  memcpy(hr, h + 8, sizeof(hr));
+  *iters_out = hs[0];
+  *relres_out = hr[1] > 0.0 ? std::sqrt(hr[0] / hr[1]) : 0.0;
+  if (hs[1] == 3) return ctx->fail(DEC_ERR_BREAKDOWN, "CG breakdown: p.Lp <= 0 or not finite");
+  if (hs[1] == 1) return ctx->fail(DEC_NOT_CONVERGED, "max_iter reached");
   return DEC_OK;
 }
 

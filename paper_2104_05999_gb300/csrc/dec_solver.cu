@@ -120,6 +120,15 @@ constexpr int kChunkL = DEC_CHUNK_L;
 // L2) and as per-phase kernels above (more warps in flight per SM: 1.5x
 // faster per iteration at 128^3).
 constexpr int64_t kPersistMaxRows = 400000;
+// FP64 solves of up to this many nodes run as one launch of a cluster of 16
+// SMs, whose 256 warps then have at most one slice each (8,192 nodes would be
+// the limit).  Measured, cluster against kernels per phase, us per solve to
+// 1e-10 with FSAI / Jacobi: 432 / 684 against 905 / 1,086 at 729 nodes, 788 /
+// 1,171 against 1,415 / 1,916 at 3,375, 1,353 / 1,762 against 1,770 / 2,245
+// at 5,832, where an iteration has grown to 24 us; the kernels need 31 at
+// 6,859 and grow no further.  A forced SELL shape keeps the kernels that have
+// shapes.
+constexpr int64_t kClusterRows = 6000;
 
 // Dynamic shared memory of a SELL kernel block and the number of its blocks:
 // one slice per warp, at most 4 resident blocks per SM (the reduction
@@ -367,44 +376,6 @@ form_T_kernel(int64_t n, const double* __restrict__ u, const double* __restrict_
     T[i] = u[i] + (tag[i] == DEC_NODE_DIRICHLET ? T0[i] : 0.0);
 }
 
-// k_eff pieces (Sec. 2.5): net outflow sum_j w_ij (T_i - T_j) of Dirichlet
-// nodes on x = 0 (q_in) and inflow on x = 1 (q_out), and the energy
-// sum over edges of w_e (T_i - T_j)^2, all with the unmodified weights.
-__global__ void __launch_bounds__(kBlock)
-k_eff_kernel(int64_t n, const int32_t* __restrict__ rowptr,
-             const int32_t* __restrict__ col, const int32_t* __restrict__ eid,
-             const int32_t* __restrict__ dpos, const uint8_t* __restrict__ tag,
-             const double* __restrict__ xyz, const double* __restrict__ w,
-             const uint8_t* __restrict__ fc, int state, const double* __restrict__ T,
-             double* out3, double* partial, unsigned* ticket) {
-  double qin = 0.0, qout = 0.0, en = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const double Ti = T[i];
-    const int32_t k0 = rowptr[i], k1 = rowptr[i + 1], kd = dpos[i];
-    double net = 0.0;
-    for (int32_t k = k0; k < k1; ++k) {
-      if (k == kd) continue;
-      const int32_t e = eid[k];
-      const double we = (int)fc[e] > state ? w[e] : 0.0;
-      const double d = Ti - T[col[k]];
-      net += we * d;
-      if (k > kd) en += we * d * d;
-    }
-    if (tag[i] == DEC_NODE_DIRICHLET) {
-      const double xi = xyz[3 * i];
-      if (xi == 0.0) qin += net;
-      else if (xi == 1.0) qout -= net;
-    }
-  }
-  double v[3] = {qin, qout, en}, t[3];
-  if (grid_reduce<kBlock, 3>(v, t, partial, ticket) && threadIdx.x == 0) {
-    out3[0] = t[0];
-    out3[1] = t[1];
-    out3[2] = t[2];
-  }
-}
-
 // Opt every staged SELL kernel into its dynamic shared memory (the FP64
 // stage of L is above the 48 KB default).
 cudaError_t init_kernel_attributes() {
@@ -425,14 +396,18 @@ cudaError_t init_kernel_attributes() {
   return e;
 }
 
-// k_eff pieces of every instance: block row blockIdx.y takes instances
+// k_eff pieces (Sec. 2.5) of every instance: net outflow sum_j w_ij (T_i - T_j)
+// of Dirichlet nodes on x = 0 (q_in), inflow on x = 1 (q_out) and the energy,
+// the sum over edges of w_e (T_i - T_j)^2, all with the unmodified weights.
+// Block row blockIdx.y takes instances
 // kKeffGroup * y ... (crack state b when `states`, Dirichlet set b when
 // `sets`, field b when `fields`), reading each row's structure and edge data
 // once for the whole group; T = u_b + T0 on Dirichlet nodes is formed on the
 // fly.  Block partials go to partial[(3 b + v) * gridDim.x + block] and
 // k_eff_batch_sum_kernel adds them in block order (deterministic).
-constexpr int kKeffGroup = 8;
-
+// kKeffGroup = 8 instances, or 1 for a single one (whose 21 idle block sums
+// took most of the 31 us at 3,375 nodes).
+template <int kKeffGroup>
 __global__ void __launch_bounds__(kBlock)
 k_eff_batch_kernel(int64_t n, int B, const int32_t* __restrict__ rowptr,
                    const int32_t* __restrict__ col, const int32_t* __restrict__ eid,
@@ -518,10 +493,12 @@ dec_status k_eff_all(dec_ctx* ctx, double* out3_host) {
   cudaStream_t s = ctx->stream;
   const unsigned G = (unsigned)std::max<int64_t>(
       1, std::min<int64_t>((n + kBlock - 1) / kBlock, (int64_t)ctx->num_sms * 4));
-  const unsigned GY = (unsigned)((B + kKeffGroup - 1) / kKeffGroup);
+  const int group = B == 1 ? 1 : 8;
+  const unsigned GY = (unsigned)((B + group - 1) / group);
+  auto kern = B == 1 ? k_eff_batch_kernel<1> : k_eff_batch_kernel<8>;
   DEC_TRY(ctx->kpartial.ensure((size_t)3 * B * G));
   DEC_TRY(ctx->out3.ensure(3 * (size_t)B + 2));
-  k_eff_batch_kernel<<<dim3(G, GY), kBlock, 0, s>>>(
+  kern<<<dim3(G, GY), kBlock, 0, s>>>(
       n, B, ctx->rowptr.p, ctx->col.p, ctx->eid.p, ctx->dpos.p, ctx->tag.p, ctx->xyz.p, ctx->w.p,
       ctx->ne, ctx->first_cut.p, ctx->n_scales > 1, ctx->n_sets > 1, ctx->n_fields > 1,
       ctx->u.p, ctx->T0.p, ctx->kpartial.p);
@@ -759,7 +736,6 @@ dec_status solve_instance(dec_ctx* ctx, int inst, double rtol, int max_iter,
   const int vs = value_set(ctx, inst);
   cudaStream_t s = ctx->stream;
   const unsigned G = (unsigned)ctx->grid_vec, Gs = (unsigned)ctx->grid_sell;
-  const SellArg<double> A64 = sell_arg(ctx->sellL, ctx->sL64.p + (int64_t)vs * ctx->sellL.total);
   const double* bvec = ctx->b.p + (int64_t)inst * n;
   double* u = ctx->u.p + (int64_t)inst * n;
   CgScalars h{};
@@ -769,6 +745,17 @@ dec_status solve_instance(dec_ctx* ctx, int inst, double rtol, int max_iter,
   dec_status st = DEC_OK;
   const bool fsai = ctx->precond == DEC_PRECOND_FSAI;
 
+  if (mode == DEC_MODE_FP64 && n <= kClusterRows && ctx->sell_force_l < 0 &&
+      ctx->sell_force_g < 0)
+    return solve_fp64_cluster(ctx, inst, rtol, max_iter, warm, iters_out, relres_out);
+  if (mode == DEC_MODE_MIXED && !warm && n <= kPersistMaxRows &&
+      (st = solve_mixed_persistent(ctx, inst, rtol, max_iter, iters_out, relres_out)) !=
+          DEC_ERR_LIMIT)
+    return st;   // the whole mixed solve ran as one cooperative kernel
+  st = DEC_OK;
+  DEC_TRY_STATUS(sell_copies(ctx, vs, mode == DEC_MODE_FP64 ? 1 : 2));
+  const SellArg<double> A64 =
+      sell_arg(ctx->sellL, ctx->sL64.p + (int64_t)vs * ctx->sellL.total);
   if (mode == DEC_MODE_FP64) {
     Ops<double, double, double> op{
         A64,
@@ -816,12 +803,7 @@ dec_status solve_instance(dec_ctx* ctx, int inst, double rtol, int max_iter,
       DEC_TRY(cudaGetLastError());
     }
     DEC_TRY(cudaMemcpyAsync(u, x, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-  } else if (mode == DEC_MODE_MIXED && !warm && n <= kPersistMaxRows &&
-             (st = solve_mixed_persistent(ctx, inst, rtol, max_iter, iters_out, relres_out)) !=
-                 DEC_ERR_LIMIT) {
-    return st;   // the whole mixed solve ran as one cooperative kernel
   } else {
-    st = DEC_OK;
     // Mixed: one FP32 PCG whose residual is replaced, every time it has
     // dropped by kSegment since the last replacement, by the FP64 residual
     // b - L x of the FP64 solution x += (FP32 accumulated update) ("reliable
@@ -906,6 +888,7 @@ dec_status time_kernel(dec_ctx* ctx, int which, int reps, size_t flush_bytes,
                        double* avg_ms) {
   const int64_t n = ctx->n;
   cudaStream_t s = ctx->stream;
+  DEC_TRY_STATUS(sell_copies(ctx, 0, 3));
   DEC_TRY(ctx->flush.ensure(flush_bytes > 0 ? flush_bytes : 1));
   for (auto* bf : {&ctx->p64, &ctx->q64, &ctx->t64, &ctx->z64, &ctx->r64}) DEC_TRY(bf->ensure(n));
   for (auto* bf : {&ctx->p32, &ctx->q32, &ctx->t32, &ctx->z32, &ctx->r32}) DEC_TRY(bf->ensure(n));

@@ -311,11 +311,38 @@ dec_status build_values(dec_ctx* ctx, int inst) {
       ctx->T0.p + (int64_t)ts * n, val, ctx->b.p + (int64_t)inst * n);
   DEC_TRY(cudaGetLastError());
   ctx->launches += 1;
-  if (inst == vs) {   // first instance of this value set: solver copies
-    const int64_t tot = ctx->sellL.total;
-    DEC_TRY_STATUS(scatter_values<double>(ctx, ctx->sellL, val, ctx->sL64.p + (int64_t)vs * tot));
-    DEC_TRY_STATUS(scatter_values<float>(ctx, ctx->sellL, val, ctx->sL32.p + (int64_t)vs * tot));
+  if (inst == vs) ctx->sell_have[vs] = 0;   // this value set's copies are stale
+  return DEC_OK;
+}
+
+dec_status sell_copies(dec_ctx* ctx, int vs, int bits) {
+  const int64_t nnz = ctx->nnz, tL = ctx->sellL.total, tlo = ctx->sellLo.total,
+                tup = ctx->sellUp.total, V = (int64_t)ctx->sell_have.size();
+  const int need = bits & ~ctx->sell_have[vs];
+  const bool fsai = ctx->precond != DEC_PRECOND_JACOBI;
+  const double* val = ctx->val64.p + vs * nnz;
+  const double* g = fsai ? ctx->g64.p + vs * nnz : nullptr;
+  if (need && !(ctx->sell_have[vs] & 1)) {   // the mixed solves need the FP64 L too
+    DEC_TRY(ctx->sL64.ensure(V * tL));
+    DEC_TRY_STATUS(scatter_values<double>(ctx, ctx->sellL, val, ctx->sL64.p + vs * tL));
   }
+  if (need & 2) {
+    DEC_TRY(ctx->sL32.ensure(V * tL));
+    DEC_TRY_STATUS(scatter_values<float>(ctx, ctx->sellL, val, ctx->sL32.p + vs * tL));
+    if (fsai) {
+      DEC_TRY(ctx->sGlo16.ensure(V * tlo));
+      DEC_TRY(ctx->sGup16.ensure(V * tup));
+      DEC_TRY_STATUS(scatter_values<__nv_bfloat16>(ctx, ctx->sellLo, g, ctx->sGlo16.p + vs * tlo));
+      DEC_TRY_STATUS(scatter_values<__nv_bfloat16>(ctx, ctx->sellUp, g, ctx->sGup16.p + vs * tup));
+    }
+  }
+  if ((need & 1) && fsai) {
+    DEC_TRY(ctx->sGlo64.ensure(V * tlo));
+    DEC_TRY(ctx->sGup64.ensure(V * tup));
+    DEC_TRY_STATUS(scatter_values<double>(ctx, ctx->sellLo, g, ctx->sGlo64.p + vs * tlo));
+    DEC_TRY_STATUS(scatter_values<double>(ctx, ctx->sellUp, g, ctx->sGup64.p + vs * tup));
+  }
+  ctx->sell_have[vs] |= need;
   return DEC_OK;
 }
 
@@ -328,10 +355,7 @@ dec_status build_values_uncracked(dec_ctx* ctx) {
       ctx->first_cut.p, -1, ctx->T0.p, ctx->val64.p, ctx->b.p);
   DEC_TRY(cudaGetLastError());
   ctx->launches += 1;
-  const int64_t tot = ctx->sellL.total;
-  DEC_TRY_STATUS(scatter_values<double>(ctx, ctx->sellL, ctx->val64.p, ctx->sL64.p));
-  DEC_TRY_STATUS(scatter_values<float>(ctx, ctx->sellL, ctx->val64.p, ctx->sL32.p));
-  (void)tot;
+  ctx->sell_have[0] = 0;
   return DEC_OK;
 }
 
@@ -374,11 +398,7 @@ dec_status build_precond(dec_ctx* ctx, int vs) {
       ctx->pos_up.p, val, g, ctx->errflag.p);
   DEC_TRY(cudaGetLastError());
   ctx->launches += 2;
-  const int64_t tlo = ctx->sellLo.total, tup = ctx->sellUp.total;
-  DEC_TRY_STATUS(scatter_values<double>(ctx, ctx->sellLo, g, ctx->sGlo64.p + (int64_t)vs * tlo));
-  DEC_TRY_STATUS(scatter_values<double>(ctx, ctx->sellUp, g, ctx->sGup64.p + (int64_t)vs * tup));
-  DEC_TRY_STATUS(scatter_values<__nv_bfloat16>(ctx, ctx->sellLo, g, ctx->sGlo16.p + (int64_t)vs * tlo));
-  DEC_TRY_STATUS(scatter_values<__nv_bfloat16>(ctx, ctx->sellUp, g, ctx->sGup16.p + (int64_t)vs * tup));
+  ctx->sell_have[vs] = 0;
   int flag = 0;
   DEC_TRY(cudaMemcpyAsync(&flag, ctx->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   DEC_TRY(cudaStreamSynchronize(s));
@@ -471,6 +491,7 @@ __global__ void fsai_rows_scatter_kernel(const int32_t* __restrict__ list,
 dec_status crack_update(dec_ctx* ctx, int64_t e) {
   cudaStream_t s = ctx->stream;
   const bool jac = ctx->precond == DEC_PRECOND_JACOBI;
+  DEC_TRY_STATUS(sell_copies(ctx, 0, 3));       // updated row by row below
   // the list holds at most 2 + deg(i) + deg(j) <= nnz rows
   DEC_TRY(ctx->big_rows.ensure(ctx->nnz + 1));
   int32_t* list = ctx->big_rows.p;
