@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 namespace dec {
@@ -32,7 +33,20 @@ namespace dec {
 namespace {
 
 constexpr int kTBlock = 256;
+constexpr int kPBlock = 1024;   // the PCG's blocks
 constexpr long kTSpinLimit = 1L << 24;
+
+// A row of the tet operator or of its factor: its four off-diagonal slots
+// side by side in [0, 4 m), its diagonal in [4 m, 5 m).  A warp reads a row
+// per lane in one 16-byte load of the columns, two of the slots and one of the
+// diagonal, all in sectors it uses fully.
+__device__ __forceinline__ void store_row(double* a, int64_t m, int64_t t, const double (&off)[4],
+                                          double diag) {
+  double2* p = reinterpret_cast<double2*>(a + 4 * t);
+  p[0] = make_double2(off[0], off[1]);
+  p[1] = make_double2(off[2], off[3]);
+  a[4 * m + t] = diag;
+}
 
 // local edge slot of the local vertex pair (a, b), a < b
 __device__ __forceinline__ int pair_slot(int a, int b) {
@@ -189,20 +203,21 @@ __global__ void mark_cut_kernel(const int32_t* __restrict__ list, int64_t nl, in
   }
 }
 
-// Row T of the two-point operator in 5 slots (slot 0 the diagonal, slot
-// v + 1 the neighbour across the face opposite vertex v, column -1 when
-// absent or when the face carries w = 0, e.g. cracked), stored slot-major
-// (k * m + T), and its right-hand side.  A tet whose faces all carry w = 0
+// Row T of the two-point operator (store_row: the diagonal, and in slot v the
+// neighbour across the face opposite vertex v, column -1 when absent or when
+// the face carries w = 0, e.g. cracked), and its right-hand side.  A tet whose faces all carry w = 0
 // becomes an identity row with rhs 0.
 __global__ void tet_rows_kernel(int64_t m, const int32_t* __restrict__ t2f,
                                 const int32_t* __restrict__ slot0,
                                 const int32_t* __restrict__ slot1, const double* __restrict__ w,
                                 const uint8_t* __restrict__ cls, const double* __restrict__ T0f,
-                                const double* __restrict__ flux, int32_t* __restrict__ col,
+                                const double* __restrict__ flux, int4* __restrict__ col,
                                 double* __restrict__ val, double* __restrict__ rhs) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m;
        t += (int64_t)gridDim.x * blockDim.x) {
-    double d = 0.0, bt = 0.0;
+    double d = 0.0, bt = 0.0, offs[4];
+    int32_t nbs[4];
+#pragma unroll
     for (int v = 0; v < 4; ++v) {
       const int32_t f = t2f[t * 4 + v];
       const double wf = w[f];
@@ -220,15 +235,15 @@ __global__ void tet_rows_kernel(int64_t m, const int32_t* __restrict__ t2f,
       } else if (flux) {
         bt -= flux[f];
       }
-      col[(int64_t)(v + 1) * m + t] = nb;
-      val[(int64_t)(v + 1) * m + t] = off;
+      nbs[v] = nb;
+      offs[v] = off;
     }
     if (d == 0.0) {
       d = 1.0;
       bt = 0.0;
     }
-    col[t] = (int32_t)t;
-    val[t] = d;
+    col[t] = make_int4(nbs[0], nbs[1], nbs[2], nbs[3]);
+    store_row(val, m, t, offs, d);
     rhs[t] = bt;
   }
 }
@@ -239,29 +254,29 @@ __global__ void tet_rows_kernel(int64_t m, const int32_t* __restrict__ t2f,
 // A[P,P] g = e_T, G_T = g / sqrt(g_T); M = G^T G.  Cholesky of the <= 5x5
 // block in FP64; a pivot <= 1e-12 max(diag) (a singular block: a group of
 // tets cut off by cracks) is factored again with that shift on the diagonal.
-// glo[k * m + T] holds G[T][col_k(T)] for the slots k whose column is T
-// (k = 0) or a lower neighbour, 0 elsewhere.
-__device__ __forceinline__ double tet_entry(const int32_t* __restrict__ col,
+// gfac's row T holds G[T][T] and, in the slots of lower neighbours c,
+// G[T][c]; 0 elsewhere.
+__device__ __forceinline__ double tet_entry(const int4* __restrict__ col,
                                             const double* __restrict__ val, int64_t m,
                                             int32_t p, int32_t q) {
-  if (p == q) return val[p];
-#pragma unroll
-  for (int k = 1; k < 5; ++k)
-    if (col[(int64_t)k * m + p] == q) return val[(int64_t)k * m + p];
-  return 0.0;
+  if (p == q) return val[4 * m + p];
+  const int4 c = col[p];
+  const int k = c.x == q ? 0 : c.y == q ? 1 : c.z == q ? 2 : c.w == q ? 3 : -1;
+  return k < 0 ? 0.0 : val[4 * (int64_t)p + k];
 }
 
-__global__ void tet_fsai_kernel(int64_t m, const int32_t* __restrict__ col,
-                                const double* __restrict__ val, double* __restrict__ glo) {
+__global__ void tet_fsai_kernel(int64_t m, const int4* __restrict__ col,
+                                const double* __restrict__ val, double* __restrict__ gfac) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m;
        t += (int64_t)gridDim.x * blockDim.x) {
     int32_t P[5];
     int slot_of[5];
     int k = 0;
-    for (int s = 1; s < 5; ++s) {
-      const int32_t c = col[(int64_t)s * m + t];
-      if (c >= 0 && c < (int32_t)t) { P[k] = c; slot_of[k] = s; ++k; }
-    }
+    const int4 c4 = col[t];
+    const int32_t cs[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+      if (cs[s] >= 0 && cs[s] < (int32_t)t) { P[k] = cs[s]; slot_of[k] = s; ++k; }
     // ascending column order, then T itself last
     for (int i = 1; i < k; ++i)
       for (int j = i; j > 0 && P[j - 1] > P[j]; --j) {
@@ -269,7 +284,6 @@ __global__ void tet_fsai_kernel(int64_t m, const int32_t* __restrict__ col,
         const int sl = slot_of[j]; slot_of[j] = slot_of[j - 1]; slot_of[j - 1] = sl;
       }
     P[k] = (int32_t)t;
-    slot_of[k] = 0;
     const int n = k + 1;
     double A[5][5];
     double dmax = 0.0;
@@ -310,27 +324,28 @@ __global__ void tet_fsai_kernel(int64_t m, const int32_t* __restrict__ col,
       g[i] = -sum / Lc[i][i];
     }
     const double scale = Lc[n - 1][n - 1];
-    for (int s = 0; s < 5; ++s) glo[(int64_t)s * m + t] = 0.0;
-    for (int i = 0; i < n; ++i) glo[(int64_t)slot_of[i] * m + t] = g[i] * scale;
+    double off[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = 0; i < n - 1; ++i) off[slot_of[i]] = g[i] * scale;
+    store_row(gfac, m, t, off, g[n - 1] * scale);
   }
 }
 
-// G^T in the same slots: gup[0] = G[T][T], gup[k] = G[c][T] for an upper
-// neighbour c of T (found in row c's slot whose column is T).
-__global__ void tet_fsai_upper_kernel(int64_t m, const int32_t* __restrict__ col,
-                                      const double* __restrict__ glo,
-                                      double* __restrict__ gup) {
+// G^T in the slots that G leaves free: slot k of an upper neighbour c gets
+// G[c][T] (found in row c's slot whose column is T; row c's lower slots are
+// not written here).  One array then serves both products.
+__global__ void tet_fsai_upper_kernel(int64_t m, const int4* __restrict__ col, double* g) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m;
        t += (int64_t)gridDim.x * blockDim.x) {
-    gup[t] = glo[t];
-    for (int s = 1; s < 5; ++s) {
-      const int32_t c = col[(int64_t)s * m + t];
-      double v = 0.0;
-      if (c > (int32_t)t) {
-        for (int k = 1; k < 5; ++k)
-          if (col[(int64_t)k * m + c] == (int32_t)t) v = glo[(int64_t)k * m + c];
-      }
-      gup[(int64_t)s * m + t] = v;
+    const int4 c4 = col[t];
+    const int32_t cs[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const int32_t c = cs[s];
+      if (c <= (int32_t)t) continue;
+      const int4 o = col[c];
+      const int32_t me = (int32_t)t;
+      const int k = o.w == me ? 3 : o.z == me ? 2 : o.y == me ? 1 : o.x == me ? 0 : -1;
+      g[4 * t + s] = k < 0 ? 0.0 : g[4 * (int64_t)c + k];
     }
   }
 }
@@ -338,45 +353,37 @@ __global__ void tet_fsai_upper_kernel(int64_t m, const int32_t* __restrict__ col
 // ------------------------------------------------------------------ PCG
 struct TetPcgArgs {
   int64_t m;
-  const int32_t* col;
-  const double* val;
+  const int4* col;          // the four neighbours, -1: none
+  const double* val;        // rows as store_row lays them out
   const double* rhs;
-  const double* glo;        // FSAI factor G (slot-major)
-  const double* gup;        // G^T in the same slots
+  const double* g;          // FSAI factor: G in the lower slots, G^T in the upper
   double* tt;               // t = G r
   double *x, *r, *p, *q;
-  double* partial;          // [2][2][grid]
-  unsigned* bar;            // [0] arrivals, [1] generation
+  double* partial;          // [2][grid]
+  unsigned* bar;            // [0] arrivals (cleared before the launch), [2] poll limit, [3] test
   int* status;              // [0] error, [1] iterations, [2] outcome
   double* result;           // [0] |b - A x|^2, [1] |b|^2
   double rtol2;
   int max_iter;
 };
 
-__device__ __forceinline__ bool tgrid_sync(unsigned* bar, int* err) {
+// Grid barrier over a counter that only grows; `target` is the arrival count
+// that lets this round pass.
+__device__ __forceinline__ bool tgrid_sync(unsigned* bar, int* err, unsigned& target) {
   __syncthreads();
+  target += gridDim.x;
   if (threadIdx.x == 0) {
-    volatile unsigned* gen = bar + 1;
-    const unsigned g = *gen;
     __threadfence();
-    const unsigned arrived = atomicAdd(bar, 1u);
-    if (arrived == gridDim.x - 1) {
-      bar[0] = 0u;
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      const unsigned lim = *(volatile unsigned*)(bar + 2);
-      const long limit = lim ? (long)lim : kTSpinLimit;
-      long polls = 0;
-      unsigned ns = 32;
-      while (*gen == g) {
-        if (++polls > limit || *(volatile int*)err) {
-          atomicExch(err, 1);
-          break;
-        }
-        __nanosleep(ns);
-        if (ns < 256) ns <<= 1;
+    atomicAdd(bar, 1u);
+    const unsigned lim = *(volatile unsigned*)(bar + 2);
+    const long limit = lim ? (long)lim : kTSpinLimit;
+    long polls = 0;
+    while ((int)(*(volatile unsigned*)bar - target) < 0) {
+      if (++polls > limit || *(volatile int*)err) {
+        atomicExch(err, 1);
+        break;
       }
+      if (polls > 16) __nanosleep(polls > 256 ? 256 : 20);
     }
     __threadfence();
   }
@@ -384,152 +391,178 @@ __device__ __forceinline__ bool tgrid_sync(unsigned* bar, int* err) {
   return *(volatile int*)err == 0;
 }
 
-// Sum of NV values over the grid, identical in every block (fixed order).
-template <int NV>
-__device__ __forceinline__ bool tgrid_sum(const double (&v)[NV], double (&tot)[NV],
-                                          double* partial, int& parity, unsigned* bar,
-                                          int* err) {
-  __shared__ double sh[kTBlock];
-  __shared__ double bc[NV];
-  double* part = partial + (size_t)parity * 2 * gridDim.x;
+// Sum of one value over the grid, identical in every block (fixed order).
+__device__ __forceinline__ bool tgrid_sum(double v, double& tot, double* partial, int& parity,
+                                          unsigned* bar, int* err, unsigned& target) {
+  __shared__ double sh[kPBlock];
+  __shared__ double bc;
+  double* part = partial + (size_t)parity * gridDim.x;
   parity ^= 1;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const double s = block_sum<kTBlock>(v[k], sh);
-    if (threadIdx.x == 0) part[k * gridDim.x + blockIdx.x] = s;
-  }
-  if (!tgrid_sync(bar, err)) return false;
+  const double s = block_sum<kPBlock>(v, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (!tgrid_sync(bar, err, target)) return false;
   if (threadIdx.x < 32) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      const double t = warp0_sum_array(part + k * gridDim.x, (int)gridDim.x);
-      if (threadIdx.x == 0) bc[k] = t;
-    }
+    const double t = warp0_sum_array(part, (int)gridDim.x);
+    if (threadIdx.x == 0) bc = t;
   }
   __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NV; ++k) tot[k] = bc[k];
-  __syncthreads();
+  tot = bc;
   return true;
 }
 
-__device__ __forceinline__ double ell_row(const TetPcgArgs& a, int64_t t, const double* x) {
-  double y = a.val[t] * x[t];
-#pragma unroll
-  for (int k = 1; k < 5; ++k) {
-    const int32_t c = a.col[k * a.m + t];
-    if (c >= 0) y = fma(a.val[k * a.m + t], x[c], y);
-  }
-  return y;
+// A row's slots and diagonal, read once a phase: kept out of L1, which the
+// operands of the gathers need, and the slots out of the way of the vectors
+// and columns (96 MB at 1.7 M rows) in L2: 111.3 against 116.0 ms for 1,084
+// iterations without the L2 hint.
+__device__ __forceinline__ void load_row(const double* M, int64_t m, int64_t t, double (&v)[4],
+                                         double& d) {
+  asm volatile("ld.global.nc.L1::no_allocate.L2::evict_first.v4.f64 {%0,%1,%2,%3}, [%4];"
+      : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(M + 4 * t));
+  asm volatile("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(d) : "l"(M + 4 * m + t));
+}
+__device__ __forceinline__ int4 load_cols(const int4* col, int64_t t) {
+  int4 c;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.s32 {%0,%1,%2,%3}, [%4];"
+      : "=r"(c.x), "=r"(c.y), "=r"(c.z), "=r"(c.w) : "l"(col + t));
+  return c;
 }
 
-// sum over the row's slots of G[k][T] x[col_k(T)] (slot 0: x[T])
-__device__ __forceinline__ double fsai_row(const TetPcgArgs& a, const double* G, int64_t t,
-                                           const double* x) {
-  double y = G[t] * x[t];
+// One phase over the rows of M: y = the diagonal times X[row] plus the sum of
+// M[row][k] X[col_k(row)] over the slots kept (PART 0: all; 1: lower columns;
+// 2: upper ones), out[row] = y, or other[row] - y for KIND 3.  Returns this
+// thread's part of the phase's sum: KIND 0: none, 1: X.y, 2: other.y,
+// 3: out.out.  The next row's columns are loaded a row ahead, so that a row's
+// values and operands come in one round trip.  Not inlined: with six copies
+// of the loop in one function their addresses spilled 1 KB of registers.
+template <int PART, int KIND>
+__device__ __noinline__ double tet_product(const int4* __restrict__ col, int64_t m,
+                                           const double* __restrict__ M, const double* X,
+                                           const double* other, double* out) {
+  const int64_t step = (int64_t)gridDim.x * kPBlock;
+  double part = 0.0;
+  int64_t t = blockIdx.x * (int64_t)kPBlock + threadIdx.x;
+  int4 next = t < m ? load_cols(col, t) : make_int4(-1, -1, -1, -1);
+  for (; t < m; t += step) {
+    const int32_t c[4] = {next.x, next.y, next.z, next.w};
+    double v[4], d, xv[4], own = 0.0;
+    bool use[4];
 #pragma unroll
-  for (int k = 1; k < 5; ++k) {
-    const int32_t c = a.col[k * a.m + t];
-    if (c >= 0) y = fma(G[k * a.m + t], x[c], y);
+    for (int k = 0; k < 4; ++k) {
+      use[k] = PART == 0 ? c[k] >= 0
+                         : PART == 1 ? (uint32_t)c[k] < (uint32_t)t : c[k] > (int32_t)t;
+      if (use[k]) xv[k] = X[c[k]];
+    }
+    load_row(M, m, t, v, d);
+    const double xt = X[t];
+    if constexpr (KIND >= 2) own = other[t];
+    if (t + step < m) next = load_cols(col, t + step);
+    double y = d * xt;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (use[k]) y = fma(v[k], xv[k], y);
+    if constexpr (KIND == 3) y = own - y;
+    out[t] = y;
+    if constexpr (KIND == 1) part = fma(xt, y, part);
+    if constexpr (KIND == 2) part = fma(own, y, part);
+    if constexpr (KIND == 3) part = fma(y, y, part);
   }
-  return y;
+  return part;
 }
 
 // PCG (FSAI M = G^T G) from x = 0 until ||b - A x|| <= rtol ||b||,
 // checked on the true residual; a recursive residual that has converged but
 // a true one that has not restarts from the true residual.  With FSAI the
 // preconditioned residual z lives in q between the update and p = z + beta p.
-__global__ void __launch_bounds__(kTBlock) tet_pcg_kernel(TetPcgArgs a) {
+// Five phases per iteration, between grid barriers, 280 B and 21 FMAs a row.
+// Bound by DRAM (103 us an iteration at 1.7 M rows: 4.6 TB/s if all of it
+// came from there) and, close behind, by the FP64 pipe (2 FMAs a clock and SM:
+// 57 us), so phases are not fused where a fused one would repeat an update
+// for every neighbour.  One block of 1,024 threads per SM: a quarter of the
+// partial sums, which every block adds up, of four blocks of 256.  The 64^3
+// cube's 1,084 iterations: 147 ms with slot-major rows, separate arrays for G
+// and G^T and four blocks of 256; 111 ms now.  More resident threads (1,536
+// or 2,048 per SM) lost 5 to 20 %, as fewer (512) did; phases in alternating
+// directions and a contiguous part of the rows per block changed nothing.
+__global__ void __launch_bounds__(kPBlock, 1) tet_pcg_kernel(TetPcgArgs a) {
   if (*(volatile unsigned*)(a.bar + 3) && blockIdx.x == gridDim.x - 1) return;
   const int64_t m = a.m;
-  const int64_t t0 = blockIdx.x * (int64_t)kTBlock + threadIdx.x;
-  const int64_t ts = (int64_t)gridDim.x * kTBlock;
+  const int64_t t0 = blockIdx.x * (int64_t)kPBlock + threadIdx.x;
+  const int64_t ts = (int64_t)gridDim.x * kPBlock;
   int* err = a.status;
   int parity = 0;
-  double v1[1], t1[1];
+  unsigned target = 0;
+  auto product = [&](auto part_c, auto kind_c, const double* M, const double* X,
+                     const double* other, double* out) {
+    return tet_product<decltype(part_c)::value, decltype(kind_c)::value>(a.col, m, M, X, other,
+                                                                         out);
+  };
+  using C0 = std::integral_constant<int, 0>;
+  using C1 = std::integral_constant<int, 1>;
+  using C2 = std::integral_constant<int, 2>;
+  using C3 = std::integral_constant<int, 3>;
+  auto sum = [&](double v, double& tot) {
+    return tgrid_sum(v, tot, a.partial, parity, a.bar, err, target);
+  };
+  // z = G^T (G r), r.z
+  auto precondition = [&](double* z, double& rz) {
+    product(C1{}, C0{}, a.g, a.r, nullptr, a.tt);
+    if (!tgrid_sync(a.bar, err, target)) return false;
+    return sum(product(C2{}, C2{}, a.g, a.tt, a.r, z), rz);
+  };
   // x = 0, r = b, |b|^2
-  double bb = 0.0;
+  double bb = 0.0, bnorm2;
   for (int64_t t = t0; t < m; t += ts) {
     const double b = a.rhs[t];
     a.x[t] = 0.0;
     a.r[t] = b;
     bb = fma(b, b, bb);
   }
-  v1[0] = bb;
-  if (!tgrid_sum<1>(v1, t1, a.partial, parity, a.bar, err)) return;
-  const double bnorm2 = t1[0];
+  if (!sum(bb, bnorm2)) return;
   const double tol2 = a.rtol2 * bnorm2;
   int it = 0, outcome = 0, restarts = 0;
   double rr_true = bnorm2;
   if (bnorm2 > 0.0) {
     for (;;) {
       // (re)start: p = z = M r, rz
-      double rz = 0.0;
-      for (int64_t t = t0; t < m; t += ts) a.tt[t] = fsai_row(a, a.glo, t, a.r);
-      if (!tgrid_sync(a.bar, err)) return;
-      for (int64_t t = t0; t < m; t += ts) {
-        const double z = fsai_row(a, a.gup, t, a.tt);
-        a.p[t] = z;
-        rz = fma(a.r[t], z, rz);
-      }
-      v1[0] = rz;
-      if (!tgrid_sum<1>(v1, t1, a.partial, parity, a.bar, err)) return;
-      rz = t1[0];
+      double rz;
+      if (!precondition(a.p, rz)) return;
       bool conv = false;
       while (it < a.max_iter) {
-        double pq = 0.0;
-        for (int64_t t = t0; t < m; t += ts) {
-          const double qt = ell_row(a, t, a.p);
-          a.q[t] = qt;
-          pq = fma(a.p[t], qt, pq);
-        }
-        v1[0] = pq;
-        if (!tgrid_sum<1>(v1, t1, a.partial, parity, a.bar, err)) return;
-        pq = t1[0];
+        double pq, rr, part = 0.0;
+        if (!sum(product(C0{}, C1{}, a.val, a.p, nullptr, a.q), pq)) return;
         if (!(pq > 0.0) || !isfinite(pq)) { outcome = 3; break; }   // breakdown
         const double alpha = rz / pq;
-        double rr = 0.0;
         for (int64_t t = t0; t < m; t += ts) {
-          a.x[t] = fma(alpha, a.p[t], a.x[t]);
           const double rt = fma(-alpha, a.q[t], a.r[t]);
           a.r[t] = rt;
-          rr = fma(rt, rt, rr);
+          part = fma(rt, rt, part);
         }
-        v1[0] = rr;
-        if (!tgrid_sum<1>(v1, t1, a.partial, parity, a.bar, err)) return;
+        if (!sum(part, rr)) return;
         ++it;
-        if (t1[0] <= tol2) { conv = true; break; }
-        // z = G^T (G r) into q, r.z
-        for (int64_t t = t0; t < m; t += ts) a.tt[t] = fsai_row(a, a.glo, t, a.r);
-        if (!tgrid_sync(a.bar, err)) return;
-        double rzf = 0.0;
-        for (int64_t t = t0; t < m; t += ts) {
-          const double z = fsai_row(a, a.gup, t, a.tt);
-          a.q[t] = z;
-          rzf = fma(a.r[t], z, rzf);
+        conv = rr <= tol2;
+        double beta = 0.0;
+        if (!conv) {
+          double rz_new;
+          if (!precondition(a.q, rz_new)) return;
+          beta = rz_new / rz;
+          rz = rz_new;
         }
-        v1[0] = rzf;
-        if (!tgrid_sum<1>(v1, t1, a.partial, parity, a.bar, err)) return;
-        const double beta = t1[0] / rz;
-        rz = t1[0];
-        for (int64_t t = t0; t < m; t += ts) a.p[t] = fma(beta, a.p[t], a.q[t]);
-        if (!tgrid_sync(a.bar, err)) return;
+        // x += alpha p here, where p is read for p = z + beta p anyway
+        for (int64_t t = t0; t < m; t += ts) {
+          const double p = a.p[t], x = a.x[t], z = a.q[t];
+          a.x[t] = fma(alpha, p, x);
+          a.p[t] = fma(beta, p, z);
+        }
+        if (!tgrid_sync(a.bar, err, target)) return;
+        if (conv) break;
       }
       // true residual r = b - A x
-      double rt2 = 0.0;
-      for (int64_t t = t0; t < m; t += ts) {
-        const double rt = a.rhs[t] - ell_row(a, t, a.x);
-        a.q[t] = rt;
-        rt2 = fma(rt, rt, rt2);
-      }
-      v1[0] = rt2;
-      if (!tgrid_sum<1>(v1, t1, a.partial, parity, a.bar, err)) return;
-      rr_true = t1[0];
+      if (!sum(product(C0{}, C3{}, a.val, a.x, a.rhs, a.q), rr_true)) return;
       if (outcome == 3) break;
       if (rr_true <= tol2) { outcome = 0; break; }
       if (!conv || ++restarts > 8) { outcome = 1; break; }   // max_iter or no progress
       for (int64_t t = t0; t < m; t += ts) a.r[t] = a.q[t];
-      if (!tgrid_sync(a.bar, err)) return;
+      if (!tgrid_sync(a.bar, err, target)) return;
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -684,11 +717,10 @@ dec_status tet_solve(dec_ctx* ctx, const double* T0_dev, double kappa, double li
   DEC_TRY(ctx->fT0.ensure(nf));
   DEC_TRY(ctx->fcls.ensure(nf));
   DEC_TRY(ctx->fcut.ensure(nf));
-  DEC_TRY(ctx->tcol.ensure(5 * m));
+  DEC_TRY(ctx->tcol.ensure(m));
   DEC_TRY(ctx->tval.ensure(5 * m));
   DEC_TRY(ctx->trhs.ensure(m));
-  DEC_TRY(ctx->tglo.ensure(5 * m));
-  DEC_TRY(ctx->tgup.ensure(5 * m));
+  DEC_TRY(ctx->tg.ensure(5 * m));
   DEC_TRY(ctx->tt.ensure(m));
   DEC_TRY(ctx->talpha.ensure(m));
   DEC_TRY(ctx->tr.ensure(m));
@@ -710,8 +742,8 @@ dec_status tet_solve(dec_ctx* ctx, const double* T0_dev, double kappa, double li
   tet_rows_kernel<<<tgrid(ctx, m), 256, 0, s>>>(m, ctx->t2f.p, ctx->fslot0.p, ctx->fslot1.p,
                                                 ctx->fw.p, ctx->fcls.p, ctx->fT0.p, flux_dev,
                                                 ctx->tcol.p, ctx->tval.p, ctx->trhs.p);
-  tet_fsai_kernel<<<tgrid(ctx, m), 256, 0, s>>>(m, ctx->tcol.p, ctx->tval.p, ctx->tglo.p);
-  tet_fsai_upper_kernel<<<tgrid(ctx, m), 256, 0, s>>>(m, ctx->tcol.p, ctx->tglo.p, ctx->tgup.p);
+  tet_fsai_kernel<<<tgrid(ctx, m), 256, 0, s>>>(m, ctx->tcol.p, ctx->tval.p, ctx->tg.p);
+  tet_fsai_upper_kernel<<<tgrid(ctx, m), 256, 0, s>>>(m, ctx->tcol.p, ctx->tg.p);
   DEC_TRY(cudaGetLastError());
   ctx->launches += 5;
   int hflag[4];
@@ -726,11 +758,11 @@ dec_status tet_solve(dec_ctx* ctx, const double* T0_dev, double kappa, double li
   DEC_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device));
   if (!coop) return ctx->fail(DEC_ERR_LIMIT, "tet_solve: cooperative launch unavailable");
   int per_sm = 0;
-  DEC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tet_pcg_kernel, kTBlock, 0));
+  DEC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tet_pcg_kernel, kPBlock, 0));
   if (per_sm < 1) return ctx->fail(DEC_ERR_LIMIT, "tet_solve: cooperative launch unavailable");
   const int grid = (int)std::max<int64_t>(
-      1, std::min<int64_t>((int64_t)ctx->num_sms * std::min(per_sm, 4), (m + kTBlock - 1) / kTBlock));
-  DEC_TRY(ctx->partial.ensure((size_t)4 * grid));
+      1, std::min<int64_t>((int64_t)ctx->num_sms, (m + kPBlock - 1) / kPBlock));
+  DEC_TRY(ctx->partial.ensure((size_t)2 * grid));
   DEC_TRY(ctx->coop.ensure(16));
   DEC_TRY(cudaMemsetAsync(ctx->coop.p, 0, 16 * sizeof(int64_t), s));
   unsigned* bar = reinterpret_cast<unsigned*>(ctx->coop.p);
@@ -740,8 +772,7 @@ dec_status tet_solve(dec_ctx* ctx, const double* T0_dev, double kappa, double li
   a.col = ctx->tcol.p;
   a.val = ctx->tval.p;
   a.rhs = ctx->trhs.p;
-  a.glo = ctx->tglo.p;
-  a.gup = ctx->tgup.p;
+  a.g = ctx->tg.p;
   a.tt = ctx->tt.p;
   a.x = ctx->talpha.p;
   a.r = ctx->tr.p;
@@ -754,7 +785,7 @@ dec_status tet_solve(dec_ctx* ctx, const double* T0_dev, double kappa, double li
   a.rtol2 = rtol * rtol;
   a.max_iter = max_iter;
   void* args[] = {&a};
-  DEC_TRY(cudaLaunchCooperativeKernel((const void*)tet_pcg_kernel, dim3(grid), dim3(kTBlock),
+  DEC_TRY(cudaLaunchCooperativeKernel((const void*)tet_pcg_kernel, dim3(grid), dim3(kPBlock),
                                       args, 0, s));
   ctx->launches += 1;
   int hs[3];
