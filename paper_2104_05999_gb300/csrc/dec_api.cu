@@ -257,7 +257,6 @@ dec_status dec_laplacian_build(dec_ctx* ctx, const double* T0, int32_t n_sets,
   const int V = shared ? 1 : std::max(ctx->n_scales, ctx->n_fields);  // value sets
   DEC_TRY(upload(ctx->T0, T0, (int64_t)n_sets * n, s));
   DEC_TRY(ctx->val64.ensure((size_t)V * nnz));
-  // the solver's copies of the values are made by the solves that use them
   ctx->sell_have.assign(V, 0);
   DEC_TRY(ctx->b.ensure((size_t)ctx->B * n));
   if (precond != DEC_PRECOND_JACOBI) {
@@ -276,7 +275,10 @@ dec_status dec_laplacian_build(dec_ctx* ctx, const double* T0, int32_t n_sets,
     DEC_TRY_STATUS(dec::batch_setup(ctx));
   } else {
     for (int inst = 0; inst < ctx->B; ++inst) DEC_TRY_STATUS(dec::build_values(ctx, inst));
-    for (int vs = 0; vs < V; ++vs) DEC_TRY_STATUS(dec::build_precond(ctx, vs));
+    for (int vs = 0; vs < V; ++vs) {
+      DEC_TRY_STATUS(dec::build_precond(ctx, vs));
+      DEC_TRY_STATUS(dec::sell_copies(ctx, vs, 3));   // the solves' copies of the values
+    }
   }
   DEC_TRY(cudaStreamSynchronize(s));
   ctx->stage = 3;

@@ -420,8 +420,9 @@ dec_status solve_mixed_persistent(dec_ctx* ctx, int inst, double rtol, int max_i
 // FP64 PCG of a small system in one launch of a thread-block cluster
 dec_status solve_fp64_cluster(dec_ctx* ctx, int inst, double rtol, int max_iter, bool warm,
                               int* iters_out, double* relres_out);
-// SELL copies of value set vs (bits 1: FP64, 2: FP32 and BF16), made on the
-// first use after a build
+// SELL copies of value set vs (bits 1: FP64, 2: FP32 and BF16), where they are
+// not up to date.  Made by the build for the single-instance solves; a batched
+// solve does not read them
 dec_status sell_copies(dec_ctx* ctx, int vs, int bits);
 dec_status batch_setup(dec_ctx* ctx);
 // warm: start every instance from the last batched solution
