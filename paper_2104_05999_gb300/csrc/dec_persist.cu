@@ -22,6 +22,7 @@
 #include <cmath>
 #include <cstring>
 #include <type_traits>
+#include <utility>
 
 namespace dec {
 
@@ -472,6 +473,9 @@ __global__ void __launch_bounds__(kCBlock, 1)
 pcg_cluster_kernel(ClusterArgs a) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
+  // No block may store into another's shared memory before that one runs:
+  // arrive here, wait after the matrix is staged, before the first sum.
+  cg::cluster_group::arrival_token started = cluster.barrier_arrive();
   __shared__ double sh[2][kCBlock];
   __shared__ double slot[2][2][kCBlocks][32];   // [parity][value][block][lane]
   __shared__ double bc[3];                      // sums and a ratio for the whole block
@@ -751,6 +755,7 @@ pcg_cluster_kernel(ClusterArgs a) {
     a.result[1] = bnorm2;
   }
   };
+  cluster.barrier_wait(std::move(started));   // every block of the cluster runs
   if (staged) run(std::true_type{});
   else run(std::false_type{});
   cluster.sync();     // no block leaves while another may write its slots
