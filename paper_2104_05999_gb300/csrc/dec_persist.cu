@@ -651,12 +651,16 @@ pcg_cluster_kernel(ClusterArgs a) {
   }
   const double bnorm2 = bc[0], tol2 = a.rtol2 * bnorm2;
   double rr = bnorm2;
-  if (a.warm && bnorm2 > 0.0) {
+  // Only b = 0, or a warm start that meets the tolerance, needs no iteration;
+  // a right-hand side that is not finite breaks down in the first one.
+  bool solved = bnorm2 == 0.0;
+  if (a.warm && !solved) {
     residual();
     rr = bc[0];
+    solved = rr <= tol2 && isfinite(bnorm2);
   }
   int iters = 0, outcome = 0;
-  while (bnorm2 > 0.0 && !(rr <= tol2)) {
+  while (!solved) {
     // (re)start: z = M r, r.z, beta = 0
     double v = 0.0;
     const double* rc = a.r[cur];
@@ -744,14 +748,14 @@ pcg_cluster_kernel(ClusterArgs a) {
     // the true residual decides
     residual();
     rr = bc[0];
-    if (breakdown) { outcome = 3; break; }
+    if (breakdown || !isfinite(bnorm2)) { outcome = 3; break; }
     if (rr <= tol2) break;
     if (iters >= a.max_iter) { outcome = 1; break; }
   }
   if (rank == 0 && threadIdx.x == 0) {
     a.status[0] = iters;
     a.status[1] = outcome;
-    a.result[0] = bnorm2 > 0.0 ? rr : 0.0;
+    a.result[0] = bnorm2 == 0.0 ? 0.0 : rr;
     a.result[1] = bnorm2;
   }
   };
