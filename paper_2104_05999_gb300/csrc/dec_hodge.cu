@@ -131,6 +131,7 @@ struct DiscGrid {
   const float* scales_f;  // [n_states], rounded
   int n_states;
   int nd;
+  bool fp32;              // radii and scales in FP32's range: sub-triangle tests in FP32
   double smax;            // largest radius scale
 };
 
@@ -191,16 +192,23 @@ __device__ __forceinline__ void pt_store(CrackPts& pts, int c, F3 v) {
 // Forms the corners from the edge vectors R (rounded once from FP64) and cT
 // (error at most eT), and bounds their error E and their size P.  With u =
 // 2^-24, l the longer side and tau = l^2 / |a x b|, the rounded circumcentre
-// of a triangle is off by at most u l (36 tau^2 + 20 tau): 12 u tau from the
-// cross product in numerator and, twice, denominator (|c| <= l tau), the rest
-// from |a|^2 b - |b|^2 a; 64 u l tau (1 + tau) is used.  Returns false when
-// the bound is too loose to be of use (thin faces).
-__device__ __forceinline__ bool crack_points(const F3 (&R)[4], F3 cT, float eT, CrackPts& pts,
+// of a triangle is off by at most u l (36 tau^2 + 24 tau): 12 u tau from the
+// cross product in numerator and, twice, denominator (|c| <= l tau), 2 u from
+// each rsqrtf, the rest from |a|^2 b - |b|^2 a; 64 u l tau (1 + tau) is used.
+// Returns false when the bound is too loose to be of use (thin faces: edges
+// of one face that differ 50-fold already are), when a corner is not finite,
+// and where the longest edge from vertex 0 is out of [1e-8, 1e8]: |a x b|^2
+// goes with l^4 and would leave FP32's normal range, which no bound here
+// covers (the FP64 test takes such tets).  Out of line: inlined, the extra
+// checks spilled 50 bytes more and 12.1 M tets with 1,500 discs took 11.2 ms
+// instead of 10.9.
+__device__ __noinline__ bool crack_points(const F3 (&R)[4], F3 cT, float eT, CrackPts& pts,
                                              float& E, float& P) {
   constexpr float kU = 5.9604645e-8f;
   float L2 = 0.0f, e = eT, p2 = dot(cT, cT);
 #pragma unroll
   for (int i = 1; i < 4; ++i) L2 = fmaxf(L2, dot(R[i], R[i]));
+  bool usable = L2 > 1e-16f && L2 < 1e16f && p2 < 1e30f;     // false for NaN, too
   pt_store(pts, 0, 0.5f * (R[0] + R[1]));
   pt_store(pts, 1, 0.5f * (R[0] + R[2]));
   pt_store(pts, 2, 0.5f * (R[0] + R[3]));
@@ -211,10 +219,12 @@ __device__ __forceinline__ bool crack_points(const F3 (&R)[4], F3 cT, float eT, 
   for (int v = 0; v < 4; ++v) {
     const F3 o = R[(v + 1) & 3], a = R[(v + 2) & 3] - o, b = R[(v + 3) & 3] - o;
     const F3 axb = cross(a, b);
-    const float aa = dot(a, a), bb = dot(b, b), nn = dot(axb, axb);
-    const F3 c = o + (0.5f / nn) * cross(aa * b - bb * a, axb);
+    const float aa = dot(a, a), bb = dot(b, b), in = rsqrtf(dot(axb, axb));
+    // the normal to unit length first: products stay below l^4
+    const F3 c = o + (0.5f * in) * cross(aa * b - bb * a, in * axb);
     pt_store(pts, 6 + v, c);
-    const float l2 = fmaxf(aa, bb), tau = l2 * rsqrtf(nn);
+    const float l2 = fmaxf(aa, bb), tau = l2 * in;
+    usable = usable && tau < 1e4f;
     // the sides a, b carry the roundings of two edge vectors (of size up to
     // sqrt(L2)) and one more
     e = fmaxf(e, 128.0f * kU * sqrtf(fmaxf(l2, L2)) * tau * (1.0f + tau));
@@ -223,7 +233,7 @@ __device__ __forceinline__ bool crack_points(const F3 (&R)[4], F3 cT, float eT, 
   pt_store(pts, 10, cT);
   P = sqrtf(fmaxf(p2, L2)) * 1.001f;
   E = e * 1.01f + 8.0f * kU * P;
-  return E < 0.02f * sqrtf(L2);        // false for NaN too
+  return usable && E < 0.02f * sqrtf(L2);
 }
 
 // The two halves of every slot's piece of dual face (below), from the edge
@@ -419,7 +429,7 @@ hodge_tet_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tet
         return cTx;
       };
       // corners of the sub-triangles: only for a tet that some disc may cut
-      int have_pts = 0;                     // 1: in pts, -1: FP64 only
+      int have_pts = grid.fp32 ? 0 : -1;    // 1: in pts, -1: FP64 only
       float Ept = 0.0f, Ppt = 0.0f;
       const double lo[3] = {cTa.x - RT, cTa.y - RT, cTa.z - RT};
       const double hi[3] = {cTa.x + RT, cTa.y + RT, cTa.z + RT};
@@ -726,6 +736,11 @@ dec_status assemble_hodge(dec_ctx* ctx, int64_t nd, bool has_k, int n_fields) {
     DEC_TRY(cudaMemcpyAsync(ctx->discs_f.p, hf.data(), sizeof(float) * hf.size(),
                             cudaMemcpyHostToDevice, s));
     g.scales_f = ctx->discs_f.p + 8 * nd;
+    // scale * r and its factors: no overflow, no underflow that matters beside
+    // corners of at least 1e-9 (those of crack_points)
+    g.fp32 = smax < 1e15;
+    for (int64_t i = 0; i < nd && g.fp32; ++i) g.fp32 = hd[7 * i + 6] < 1e15;
+    g.fp32 = g.fp32 && hs.front() > 1e-15;
     g.discs_f = reinterpret_cast<const float4*>(ctx->discs_f.p);
     double lo[3] = {0, 0, 0}, hi[3] = {1, 1, 1}, rmax = 0;
     for (int64_t i = 0; i < nd; ++i) {
