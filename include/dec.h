@@ -181,7 +181,8 @@ enum {
  * dec_hodge_assemble and dec_hodge_assemble_fields calls of the context.
  * DEC_GEOM_MIXED computes a tet in FP32 when L^3 <= 16 |6 V| (L its longest
  * edge from its first vertex, V its volume; a regular tet has
- * L^3 / |6 V| = 2.8, a Kuhn tet 5.2), in FP64 otherwise.  Crack decisions
+ * L^3 / |6 V| = 2.8, a Kuhn tet 5.2) and L lies in [1e-7, 1e7], in FP64
+ * otherwise.  Crack decisions
  * are those of the FP64 geometry: the FP32 circumcentre only serves as a
  * filter with an error bound, and any tet that a disc may cut has its
  * circumcentre formed again in FP64 for the exact test.  The FP32 pieces

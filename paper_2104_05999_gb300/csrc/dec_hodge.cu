@@ -312,11 +312,13 @@ __device__ __forceinline__ void tet_pieces(const Vec3<T> (&R)[4], Vec3<T>& cT, T
   slot(5, 2, 3, 0, 1);
 }
 
-// Shape bound of the FP32 geometry (DEC_GEOM_MIXED): a tet is computed in
-// FP32 when L^3 <= kShapeMax |6 V|, L the longest of its edges from vertex 0
-// (a regular tet has 2.8, a Kuhn tet 5.2; 96 % of the tets of a jittered
-// Delaunay cube pass 16), in FP64 otherwise.
+// Bounds of the FP32 geometry (DEC_GEOM_MIXED): a tet is computed in FP32
+// when L^3 <= kShapeMax |6 V|, L the longest of its edges from vertex 0 (a
+// regular tet has 2.8, a Kuhn tet 5.2; 96 % of the tets of a jittered Delaunay
+// cube pass 16), and L lies in [1e-7, 1e7], where fourth powers of lengths and
+// their inverses stay in FP32's normal range; in FP64 otherwise.
 constexpr float kShapeMax = 16.0f;
+constexpr float kMinEdge2 = 1e-14f, kMaxEdge2 = 1e14f;
 
 // MIXED = false: every tet in FP64.  MIXED = true: well-shaped tets in FP32.
 // n_fp64 counts the tets computed in FP64.
@@ -356,7 +358,7 @@ hodge_tet_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tet
       const float det6 = fabsf(dot(Rf[1], cross(Rf[2], Rf[3])));
       const float L2 = fmaxf(dot(Rf[1], Rf[1]), fmaxf(dot(Rf[2], Rf[2]), dot(Rf[3], Rf[3])));
       const float L = sqrtf(L2);
-      if (L2 * L <= kShapeMax * det6) {
+      if (L2 * L <= kShapeMax * det6 && L2 > kMinEdge2 && L2 < kMaxEdge2) {
         fast = true;
         F3 cTf;
         float b0[6], b1[6];

@@ -79,3 +79,21 @@ def test_states_of_unlike_sizes(cube, name):
         scales = scales * 1e39
     want = oracle_states(xyz, tets, discs, scales)
     assert np.array_equal(states(xyz, tets, discs, scales), want)
+
+
+@pytest.mark.parametrize("power", POWERS)
+def test_fp32_geometry_in_any_unit(cube, power):
+    """DEC_GEOM_MIXED: the same states, and *1 within the 2e-6 of the largest
+    weight that FP32 geometry is held to at unit scale."""
+    xyz, tets, discs, scales, want = cube
+    x, d = scaled(xyz, discs, 2.0 ** power)
+    assert np.array_equal(states(x, tets, d, scales, geom=1), want)
+    from paper_2104_05999_gb300 import abi
+    E, t2e = O.edge_list(tets)
+    w = O.hodge_star1(xyz, tets, E, t2e) * 2.0 ** power
+    with abi.Context(device=0) as ctx:
+        ctx.dec_set_geom_precision(abi.DEC_GEOM_MIXED)
+        ctx.dec_mesh_upload(np.ascontiguousarray(x), tets, np.zeros(len(x), dtype=np.uint8))
+        ctx.dec_hodge_assemble(None)
+        got = ctx.dec_get_hodge()[0]
+    assert np.abs(got - w).max() <= 2e-6 * np.abs(w).max()
