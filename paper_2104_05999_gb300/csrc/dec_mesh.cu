@@ -39,8 +39,9 @@ __device__ __forceinline__ float trunc_f32(double v) {
 // truncated coordinates move each difference by at most 2^-22 S + 2^-24 D, so
 // the determinant of the FP32 differences is off by less than
 // 64 2^-22 S D^2 (18 D^2 times that shift, plus 24 2^-24 D^3 for its own
-// roundings, D <= 2 S).  The FP64 determinant (0.5 ms for 12 M tets: the FP64
-// pipe) decides the rest.
+// roundings, D <= 2 S).  Underflow adds at most 1e-44 (1 + D), nothing beside
+// a bound in the normal range (which D > 1e-18 with it).  The FP64 determinant
+// (0.5 ms for 12 M tets: the FP64 pipe) decides the rest.
 __device__ __forceinline__ bool tet_positive(const double* __restrict__ xyz, int4 v) {
   const double* p[4] = {xyz + 3 * (int64_t)v.x, xyz + 3 * (int64_t)v.y, xyz + 3 * (int64_t)v.z,
                         xyz + 3 * (int64_t)v.w};
@@ -65,7 +66,8 @@ __device__ __forceinline__ bool tet_positive(const double* __restrict__ xyz, int
   const float det = d[0][0] * (d[1][1] * d[2][2] - d[1][2] * d[2][1]) +
                     d[0][1] * (d[1][2] * d[2][0] - d[1][0] * d[2][2]) +
                     d[0][2] * (d[1][0] * d[2][1] - d[1][1] * d[2][0]);
-  if (S < 1e12f && S > 1e-12f && det > 1.6e-5f * S * (D * D)) return true;
+  const float bound = 1.6e-5f * S * (D * D);
+  if (S < 1e12f && S > 1e-12f && bound > 1.2e-38f && det > bound) return true;
   const double ax = c[1][0] - c[0][0], ay = c[1][1] - c[0][1], az = c[1][2] - c[0][2];
   const double bx = c[2][0] - c[0][0], by = c[2][1] - c[0][1], bz = c[2][2] - c[0][2];
   const double cx = c[3][0] - c[0][0], cy = c[3][1] - c[0][1], cz = c[3][2] - c[0][2];
