@@ -240,9 +240,10 @@ dec_status dec_k_eff(dec_ctx* ctx, double* q_in, double* q_out, double* energy);
 
 /* Launch shape the last DEC_MODE_MIXED_BATCHED solve of this context used,
  * as picked by its autotuner: the first batched solve of a problem size
- * (nodes, matrix entries) at each instance stride (8, 16, 32, 64) times a
- * few iterations of every variant and keeps the fastest for the context's
- * later solves of that size.
+ * (nodes, matrix entries) with each kind of instances (Dirichlet sets, crack
+ * states, conductivity fields) at each instance stride (8, 16, 32, 64) times
+ * a few iterations of every variant and keeps the fastest for the context's
+ * later solves of that size and kind.
  *   gather_entries  host: 1000 * K / 8 (K = matrix entries per chunk of a
  *                   warp's structure staged in shared memory; Dirichlet
  *                   sets of 8 or 16 instances only) + 100 * (gathers into

@@ -1839,15 +1839,17 @@ dec_status solve_batched(dec_ctx* ctx, double rtol, int max_iter, int* iters,
     ctx->launches += 1;
     return e;
   };
-  // Autotuner: the first batched solve of a problem size at this instance
-  // stride times kTuneIters FP32 iterations of every variant and keeps the
-  // fastest.  All variants give bit-identical results.
+  // Autotuner: the first batched solve of a problem size with this kind of
+  // instances at this stride times kTuneIters FP32 iterations of every
+  // variant and keeps the fastest.  All variants give bit-identical results.
   int slot = 0;
   while ((8 << slot) < BS) ++slot;
   // the choice is kept for later solves of a problem of the same size (the
-  // same mesh uploaded again, as a benchmark or a time loop does)
-  const bool same = ctx->batch_tune_key[slot][0] == n && ctx->batch_tune_key[slot][1] == ctx->nnz;
-  int v = same ? ctx->batch_variant[slot] - 1 : -1;
+  // same mesh uploaded again, as a benchmark or a time loop does) and kind:
+  // other kinds run other kernels, and only Dirichlet sets have the staged ones
+  int64_t* key = ctx->batch_tune_key[kind][slot];
+  const bool same = key[0] == n && key[1] == ctx->nnz;
+  int v = same ? ctx->batch_variant[kind][slot] - 1 : -1;
   if (ctx->batch_force != 0) {
     // a variant chosen by the caller (dec_set_batch_variant): no tuning
     v = -1;
@@ -1884,9 +1886,9 @@ dec_status solve_batched(dec_ctx* ctx, double rtol, int max_iter, int* iters,
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    ctx->batch_variant[slot] = v + 1;
-    ctx->batch_tune_key[slot][0] = n;
-    ctx->batch_tune_key[slot][1] = ctx->nnz;
+    ctx->batch_variant[kind][slot] = v + 1;
+    key[0] = n;
+    key[1] = ctx->nnz;
   }
   ctx->batch_variant_used = kGatherVariants[v];
   // device time of the solve's launch (dec_get_batch_kernel_ms)

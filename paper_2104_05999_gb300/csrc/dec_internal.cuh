@@ -179,8 +179,8 @@ struct dec_ctx {
   dec::DevBuf<__nv_bfloat16> bGloB, bGupB;     // per-instance halves [total][BS]
   dec::DevBuf<double> bb, bx64, br64, bpartial;
   dec::DevBuf<int64_t> crack_buf;          // crack growth: block bests, picked edge
-  int batch_variant[4] = {0, 0, 0, 0};     // tuned variant + 1 per stride 8..64
-  int64_t batch_tune_key[4][2] = {};       // (n, nnz) each choice was tuned for
+  int batch_variant[3][4] = {};            // tuned variant + 1 per kind and stride 8..64
+  int64_t batch_tune_key[3][4][2] = {};    // (n, nnz) each choice was tuned for
   int batch_variant_used = -1;             // variant of the last batched solve
   int batch_force = 0;                     // dec_set_batch_variant (0: autotune)
   // launch shapes of the single-instance SELL kernels per precision
