@@ -144,6 +144,7 @@ struct dec_ctx {
   // solver state
   dec::DevBuf<double> x64, r64, z64, p64, q64, t64, u;  // u: [B][n] result
   dec::DevBuf<double> p64b, r64b;  // second buffers of p and r
+  int cluster_fits[2] = {-1, -1};  // Jacobi, FSAI: 1 if a cluster can be placed, -1 unknown
   dec::DevBuf<float> x32, r32, z32, p32, q32, t32, r32b, p32b;
   dec::DevBuf<double> partial;     // [kRedSlots][reduce_grid]
   dec::DevBuf<unsigned> ticket;
@@ -417,7 +418,8 @@ dec_status k_eff_all(dec_ctx* ctx, double* out3_host);   // [B][3], one pass
 dec_status form_T(dec_ctx* ctx, int inst, double* T);
 dec_status solve_mixed_persistent(dec_ctx* ctx, int inst, double rtol, int max_iter,
                                   int* iters_out, double* relres_out);
-// FP64 PCG of a small system in one launch of a thread-block cluster
+// FP64 PCG of a small system in one launch of a thread-block cluster;
+// DEC_ERR_LIMIT, with nothing done, where the device cannot place the cluster
 dec_status solve_fp64_cluster(dec_ctx* ctx, int inst, double rtol, int max_iter, bool warm,
                               int* iters_out, double* relres_out);
 // SELL copies of value set vs (bits 1: FP64, 2: FP32 and BF16), where they are

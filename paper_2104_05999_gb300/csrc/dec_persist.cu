@@ -771,6 +771,35 @@ dec_status solve_fp64_cluster(dec_ctx* ctx, int inst, double rtol, int max_iter,
   const int vs = value_set(ctx, inst);
   cudaStream_t s = ctx->stream;
   const bool fsai = ctx->precond == DEC_PRECOND_FSAI;
+  const int cap = 19 * 1024;  // 190 KB of values and 16-bit columns
+  const int smem = cap * (int)(sizeof(double) + sizeof(uint16_t));
+  auto kern = fsai ? pcg_cluster_kernel<false> : pcg_cluster_kernel<true>;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kCBlocks;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kCBlocks);
+  cfg.blockDim = dim3(kCBlock);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  // 16 blocks are above the portable cluster size: a device (or a part of
+  // one) whose GPCs have fewer SMs to give cannot place such a cluster
+  int& fits = ctx->cluster_fits[fsai];
+  if (fits < 0) {
+    int clusters = 0;
+    const bool ok =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
+            cudaSuccess &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+            cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    fits = ok && clusters > 0 ? 1 : 0;
+  }
+  if (!fits) return DEC_ERR_LIMIT;
   DEC_TRY_STATUS(sell_copies(ctx, vs, 1));
   DEC_TRY(ctx->coop.ensure(16));
   DEC_TRY(ctx->p64b.ensure(n));
@@ -795,22 +824,7 @@ dec_status solve_fp64_cluster(dec_ctx* ctx, int inst, double rtol, int max_iter,
   a.warm = warm ? 1 : 0;
   a.status = reinterpret_cast<int*>(ctx->coop.p + 2);
   a.result = reinterpret_cast<double*>(ctx->coop.p + 8);
-  a.cap = 19 * 1024;          // 190 KB of values and 16-bit columns
-  const int smem = a.cap * (int)(sizeof(double) + sizeof(uint16_t));
-  auto kern = fsai ? pcg_cluster_kernel<false> : pcg_cluster_kernel<true>;
-  DEC_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  DEC_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = kCBlocks;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(kCBlocks);
-  cfg.blockDim = dim3(kCBlock);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  a.cap = cap;
   DEC_TRY(cudaLaunchKernelEx(&cfg, kern, a));
   DEC_TRY(cudaGetLastError());
   ctx->launches += 1;

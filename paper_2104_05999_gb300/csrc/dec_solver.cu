@@ -746,8 +746,10 @@ dec_status solve_instance(dec_ctx* ctx, int inst, double rtol, int max_iter,
   const bool fsai = ctx->precond == DEC_PRECOND_FSAI;
 
   if (mode == DEC_MODE_FP64 && n <= kClusterRows && ctx->sell_force_l < 0 &&
-      ctx->sell_force_g < 0)
-    return solve_fp64_cluster(ctx, inst, rtol, max_iter, warm, iters_out, relres_out);
+      ctx->sell_force_g < 0 &&
+      (st = solve_fp64_cluster(ctx, inst, rtol, max_iter, warm, iters_out, relres_out)) !=
+          DEC_ERR_LIMIT)
+    return st;   // (the kernels per phase where no such cluster can be placed)
   if (mode == DEC_MODE_MIXED && !warm && n <= kPersistMaxRows &&
       (st = solve_mixed_persistent(ctx, inst, rtol, max_iter, iters_out, relres_out)) !=
           DEC_ERR_LIMIT)
