@@ -33,7 +33,12 @@ namespace dec {
 namespace {
 
 constexpr int kTBlock = 256;
-constexpr int kPBlock = 1024;   // the PCG's blocks
+// The PCG's blocks, one per SM: 1,024 threads, or 256 while a thread then has
+// at most kPSmallRows rows.  Sums over a block and its barriers cost a small
+// solve more than rows in flight gain: ms with 256 against 1,024 threads, 1.03
+// and 1.47 at 179 rows, 5.90 and 8.79 at 23,006, 11.2 and 13.9 at 82,993, 19.0
+// and 22.7 at 203,530 (5.2 rows a thread), 38.5 and 35.1 at 405,273.
+constexpr int kPBlock = 1024, kPSmall = 256, kPSmallRows = 6;
 constexpr long kTSpinLimit = 1L << 24;
 
 // A row of the tet operator or of its factor: its four off-diagonal slots
@@ -392,13 +397,14 @@ __device__ __forceinline__ bool tgrid_sync(unsigned* bar, int* err, unsigned& ta
 }
 
 // Sum of one value over the grid, identical in every block (fixed order).
+template <int BLOCK>
 __device__ __forceinline__ bool tgrid_sum(double v, double& tot, double* partial, int& parity,
                                           unsigned* bar, int* err, unsigned& target) {
-  __shared__ double sh[kPBlock];
+  __shared__ double sh[BLOCK];
   __shared__ double bc;
   double* part = partial + (size_t)parity * gridDim.x;
   parity ^= 1;
-  const double s = block_sum<kPBlock>(v, sh);
+  const double s = block_sum<BLOCK>(v, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = s;
   if (!tgrid_sync(bar, err, target)) return false;
   if (threadIdx.x < 32) {
@@ -434,13 +440,13 @@ __device__ __forceinline__ int4 load_cols(const int4* col, int64_t t) {
 // 3: out.out.  The next row's columns are loaded a row ahead, so that a row's
 // values and operands come in one round trip.  Not inlined: with six copies
 // of the loop in one function their addresses spilled 1 KB of registers.
-template <int PART, int KIND>
+template <int BLOCK, int PART, int KIND>
 __device__ __noinline__ double tet_product(const int4* __restrict__ col, int64_t m,
                                            const double* __restrict__ M, const double* X,
                                            const double* other, double* out) {
-  const int64_t step = (int64_t)gridDim.x * kPBlock;
+  const int64_t step = (int64_t)gridDim.x * BLOCK;
   double part = 0.0;
-  int64_t t = blockIdx.x * (int64_t)kPBlock + threadIdx.x;
+  int64_t t = blockIdx.x * (int64_t)BLOCK + threadIdx.x;
   int4 next = t < m ? load_cols(col, t) : make_int4(-1, -1, -1, -1);
   for (; t < m; t += step) {
     const int32_t c[4] = {next.x, next.y, next.z, next.w};
@@ -477,31 +483,32 @@ __device__ __noinline__ double tet_product(const int4* __restrict__ col, int64_t
 // Bound by DRAM (103 us an iteration at 1.7 M rows: 4.6 TB/s if all of it
 // came from there) and, close behind, by the FP64 pipe (2 FMAs a clock and SM:
 // 57 us), so phases are not fused where a fused one would repeat an update
-// for every neighbour.  One block of 1,024 threads per SM: a quarter of the
+// for every neighbour.  One block per SM: at 1,024 threads a quarter of the
 // partial sums, which every block adds up, of four blocks of 256.  The 64^3
 // cube's 1,084 iterations: 147 ms with slot-major rows, separate arrays for G
 // and G^T and four blocks of 256; 111 ms now.  More resident threads (1,536
 // or 2,048 per SM) lost 5 to 20 %, as fewer (512) did; phases in alternating
 // directions and a contiguous part of the rows per block changed nothing.
-__global__ void __launch_bounds__(kPBlock, 1) tet_pcg_kernel(TetPcgArgs a) {
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK, 1) tet_pcg_kernel(TetPcgArgs a) {
   if (*(volatile unsigned*)(a.bar + 3) && blockIdx.x == gridDim.x - 1) return;
   const int64_t m = a.m;
-  const int64_t t0 = blockIdx.x * (int64_t)kPBlock + threadIdx.x;
-  const int64_t ts = (int64_t)gridDim.x * kPBlock;
+  const int64_t t0 = blockIdx.x * (int64_t)BLOCK + threadIdx.x;
+  const int64_t ts = (int64_t)gridDim.x * BLOCK;
   int* err = a.status;
   int parity = 0;
   unsigned target = 0;
   auto product = [&](auto part_c, auto kind_c, const double* M, const double* X,
                      const double* other, double* out) {
-    return tet_product<decltype(part_c)::value, decltype(kind_c)::value>(a.col, m, M, X, other,
-                                                                         out);
+    return tet_product<BLOCK, decltype(part_c)::value, decltype(kind_c)::value>(a.col, m, M, X,
+                                                                                other, out);
   };
   using C0 = std::integral_constant<int, 0>;
   using C1 = std::integral_constant<int, 1>;
   using C2 = std::integral_constant<int, 2>;
   using C3 = std::integral_constant<int, 3>;
   auto sum = [&](double v, double& tot) {
-    return tgrid_sum(v, tot, a.partial, parity, a.bar, err, target);
+    return tgrid_sum<BLOCK>(v, tot, a.partial, parity, a.bar, err, target);
   };
   // z = G^T (G r), r.z
   auto precondition = [&](double* z, double& rz) {
@@ -757,11 +764,15 @@ dec_status tet_solve(dec_ctx* ctx, const double* T0_dev, double kappa, double li
   int coop = 0;
   DEC_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device));
   if (!coop) return ctx->fail(DEC_ERR_LIMIT, "tet_solve: cooperative launch unavailable");
+  const bool small = m <= (int64_t)kPSmall * kPSmallRows * ctx->num_sms;
+  const int block = small ? kPSmall : kPBlock;
+  const void* kern = small ? (const void*)tet_pcg_kernel<kPSmall>
+                           : (const void*)tet_pcg_kernel<kPBlock>;
   int per_sm = 0;
-  DEC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tet_pcg_kernel, kPBlock, 0));
+  DEC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, 0));
   if (per_sm < 1) return ctx->fail(DEC_ERR_LIMIT, "tet_solve: cooperative launch unavailable");
   const int grid = (int)std::max<int64_t>(
-      1, std::min<int64_t>((int64_t)ctx->num_sms, (m + kPBlock - 1) / kPBlock));
+      1, std::min<int64_t>((int64_t)ctx->num_sms, (m + block - 1) / block));
   DEC_TRY(ctx->partial.ensure((size_t)2 * grid));
   DEC_TRY(ctx->coop.ensure(16));
   DEC_TRY(cudaMemsetAsync(ctx->coop.p, 0, 16 * sizeof(int64_t), s));
@@ -785,8 +796,7 @@ dec_status tet_solve(dec_ctx* ctx, const double* T0_dev, double kappa, double li
   a.rtol2 = rtol * rtol;
   a.max_iter = max_iter;
   void* args[] = {&a};
-  DEC_TRY(cudaLaunchCooperativeKernel((const void*)tet_pcg_kernel, dim3(grid), dim3(kPBlock),
-                                      args, 0, s));
+  DEC_TRY(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(block), args, 0, s));
   ctx->launches += 1;
   int hs[3];
   double hr[2];
