@@ -119,6 +119,8 @@ __device__ __noinline__ double crack_rho_s(V3 P0, V3 P1, V3 P2, double s0, doubl
   return sqrt(dot(g, g));
 }
 
+constexpr float kU = 5.9604645e-8f;    // 2^-24, the rounding unit of FP32
+
 struct DiscGrid {
   double lo[3];
   double inv_cell;
@@ -204,7 +206,6 @@ __device__ __forceinline__ void pt_store(CrackPts& pts, int c, F3 v) {
 // instead of 10.9.
 __device__ __noinline__ bool crack_points(const F3 (&R)[4], F3 cT, float eT, CrackPts& pts,
                                              float& E, float& P) {
-  constexpr float kU = 5.9604645e-8f;
   float L2 = 0.0f, e = eT, p2 = dot(cT, cT);
 #pragma unroll
   for (int i = 1; i < 4; ++i) L2 = fmaxf(L2, dot(R[i], R[i]));
@@ -312,6 +313,73 @@ __device__ __forceinline__ void tet_pieces(const Vec3<T> (&R)[4], Vec3<T>& cT, T
   slot(5, 2, 3, 0, 1);
 }
 
+// The ball test is conservative (the in-plane reach is bounded by
+// r + R_T).  Most candidate discs are far from the tet, and GB300's FP64 pipe is
+// narrow, so the two rejections are first made entirely in FP32 from
+// c_T rounded once per tet and the discs rounded once on the host.
+// With u = 2^-24 and S = A_t + A_d (bounds on |c_T| and |centre| per
+// coordinate), the offset v = c_T - centre carries an error of at most
+// 2uS per coordinate, so (first order, |normal| = 1):
+//   |dp32 - dp| <= 6 sqrt(3) u S,   |par32 - par| <= 63 u S^2
+// (dp the distance to the disc plane, par = |v|^2 - dp^2).  The
+// margins below are twice these plus the roundings of the thresholds,
+// so FP32 rejects only where the FP64 test rejects too: the decisions,
+// and so *1 and the crack states, are unchanged.
+struct BallF {
+  float x, y, z;    // centre
+  float A, R;       // bound on the centre's coordinates, radius rounded up
+};
+__device__ __forceinline__ BallF ball_f32(V3 c, double R) {
+  BallF b{(float)c.x, (float)c.y, (float)c.z, 0.0f, (float)R * (1.0f + 4.0f * kU)};
+  b.A = fmaxf(fabsf(b.x), fmaxf(fabsf(b.y), fabsf(b.z))) * (1.0f + 2.0f * kU);
+  return b;
+}
+__device__ __forceinline__ bool ball_meets_disc(const DiscGrid& grid, const BallF& b, int id) {
+  const float4 d0 = __ldg(grid.discs_f + 2 * (int64_t)id);
+  const float4 d1 = __ldg(grid.discs_f + 2 * (int64_t)id + 1);
+  const float vx = b.x - d0.x, vy = b.y - d0.y, vz = b.z - d0.z;
+  const float S = b.A + d0.w;
+  const float dpf = fmaf(vx, d1.x, fmaf(vy, d1.y, vz * d1.z));
+  if (fabsf(dpf) > b.R + (24.0f * S + 8.0f * b.R) * kU) return false;   // ball misses the plane
+  const float vv = fmaf(vx, vx, fmaf(vy, vy, vz * vz));
+  const float par = fmaf(-dpf, dpf, vv);
+  const float T = d1.w + b.R;
+  return !(par > T * T * (1.0f + 8.0f * kU) + 128.0f * kU * S * S);     // else misses the disc
+}
+
+// test(id) for every disc whose cells the box of the ball (c, R) meets
+template <typename Test>
+__device__ __forceinline__ void for_candidates(const DiscGrid& grid, V3 c, double R, Test&& test) {
+  const double lo[3] = {c.x - R, c.y - R, c.z - R};
+  const double hi[3] = {c.x + R, c.y + R, c.z + R};
+  int c0[3], c1[3];
+  bool empty = false;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    double f0 = (lo[d] - grid.lo[d]) * grid.inv_cell;
+    double f1 = (hi[d] - grid.lo[d]) * grid.inv_cell;
+    if (f1 < 0.0 || f0 >= (double)grid.dim[d]) empty = true;
+    c0[d] = (int)fmax(0.0, floor(f0));
+    c1[d] = (int)fmin((double)grid.dim[d] - 1.0, floor(f1));
+  }
+  if (empty) return;
+  const int64_t ncell = (int64_t)(c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) *
+                        (c1[2] - c0[2] + 1);
+  // a far circumcentre (flat boundary tet): fewer tests without the
+  // grid, i.e. every disc once (one pass of the loops below); one call
+  // site of test keeps the kernel small
+  const bool all = ncell > grid.nd;
+  if (all) c1[0] = c0[0], c1[1] = c0[1], c1[2] = c0[2];
+  for (int gz = c0[2]; gz <= c1[2]; ++gz)
+    for (int gy = c0[1]; gy <= c1[1]; ++gy)
+      for (int gx = c0[0]; gx <= c1[0]; ++gx) {
+        const int cell = gx + grid.dim[0] * (gy + grid.dim[1] * gz);
+        const int i0 = all ? 0 : grid.start[cell];
+        const int i1 = all ? grid.nd : grid.start[cell + 1];
+        for (int it = i0; it < i1; ++it) test(all ? it : grid.items[it]);
+      }
+}
+
 // Bounds of the FP32 geometry (DEC_GEOM_MIXED): a tet is computed in FP32
 // when L^3 <= kShapeMax |6 V|, L the longest of its edges from vertex 0 (a
 // regular tet has 2.8, a Kuhn tet 5.2; 96 % of the tets of a jittered Delaunay
@@ -321,14 +389,16 @@ constexpr float kShapeMax = 16.0f;
 constexpr float kMinEdge2 = 1e-14f, kMaxEdge2 = 1e14f;
 
 // MIXED = false: every tet in FP64.  MIXED = true: well-shaped tets in FP32.
-// n_fp64 counts the tets computed in FP64.
+// n_fp64 counts the tets computed in FP64, n_thin those left to
+// crack_thin_kernel (thin: 2 * tet + FP32 geometry, in any order).
 template <bool MIXED>
 __global__ void __launch_bounds__(kHodgeThreads, 3)
 hodge_tet_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tets,
                  const double* __restrict__ kcond, int64_t m,
                  double* __restrict__ piece, double* __restrict__ kpart,
                  uint8_t* __restrict__ slot_cut, DiscGrid grid,
-                 unsigned long long* __restrict__ n_fp64) {
+                 unsigned long long* __restrict__ n_fp64, unsigned long long* __restrict__ n_thin,
+                 uint32_t* __restrict__ thin) {
   __shared__ CrackPts pts;
   unsigned n64 = 0;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m;
@@ -431,55 +501,18 @@ hodge_tet_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tet
         return cTx;
       };
       // corners of the sub-triangles: only for a tet that some disc may cut
-      int have_pts = grid.fp32 ? 0 : -1;    // 1: in pts, -1: FP64 only
+      int have_pts = 0;                     // 1: in pts, -1: FP64 only
       float Ept = 0.0f, Ppt = 0.0f;
-      const double lo[3] = {cTa.x - RT, cTa.y - RT, cTa.z - RT};
-      const double hi[3] = {cTa.x + RT, cTa.y + RT, cTa.z + RT};
-      int c0[3], c1[3];
-      bool empty = false;
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        double f0 = (lo[d] - grid.lo[d]) * grid.inv_cell;
-        double f1 = (hi[d] - grid.lo[d]) * grid.inv_cell;
-        if (f1 < 0.0 || f0 >= (double)grid.dim[d]) empty = true;
-        c0[d] = (int)fmax(0.0, floor(f0));
-        c1[d] = (int)fmin((double)grid.dim[d] - 1.0, floor(f1));
-      }
-      // The ball test is conservative (the in-plane reach is bounded by
-      // r + R_T).  Most candidate discs are far from the tet, and GB300's FP64 pipe is
-      // narrow, so the two rejections are first made entirely in FP32 from
-      // c_T rounded once per tet and the discs rounded once on the host.
-      // With u = 2^-24 and S = A_t + A_d (bounds on |c_T| and |centre| per
-      // coordinate), the offset v = c_T - centre carries an error of at most
-      // 2uS per coordinate, so (first order, |normal| = 1):
-      //   |dp32 - dp| <= 6 sqrt(3) u S,   |par32 - par| <= 63 u S^2
-      // (dp the distance to the disc plane, par = |v|^2 - dp^2).  The
-      // margins below are twice these plus the roundings of the thresholds,
-      // so FP32 rejects only where the FP64 test rejects too: the decisions,
-      // and so *1 and the crack states, are unchanged.
-      constexpr float kU = 5.9604645e-8f;    // 2^-24
-      const float Cx = (float)cTa.x, Cy = (float)cTa.y, Cz = (float)cTa.z;
-      const float At = fmaxf(fabsf(Cx), fmaxf(fabsf(Cy), fabsf(Cz))) * (1.0f + 2.0f * kU);
-      const float RTf = (float)RT * (1.0f + 4.0f * kU);
+      const BallF ball = ball_f32(cTa, RT);
       auto test_disc = [&](int id) {
-        {
-          const float4 d0 = __ldg(grid.discs_f + 2 * (int64_t)id);
-          const float4 d1 = __ldg(grid.discs_f + 2 * (int64_t)id + 1);
-          const float vx = Cx - d0.x, vy = Cy - d0.y, vz = Cz - d0.z;
-          const float S = At + d0.w;
-          const float dpf = fmaf(vx, d1.x, fmaf(vy, d1.y, vz * d1.z));
-          if (fabsf(dpf) > RTf + (24.0f * S + 8.0f * RTf) * kU) return;   // ball misses the plane
-          const float vv = fmaf(vx, vx, fmaf(vy, vy, vz * vz));
-          const float par = fmaf(-dpf, dpf, vv);
-          const float T = d1.w + RTf;
-          if (par > T * T * (1.0f + 8.0f * kU) + 128.0f * kU * S * S) return;   // misses the disc
-        }
+        if (have_pts < 0 || !ball_meets_disc(grid, ball, id)) return;
         // The sub-triangles are then tested in FP32 on corners relative to
         // vertex 0, with bounds on every step's error, and in FP64 only where
         // a bound leaves the answer open (about 1 % of the pairs of tet and
         // disc that come this far): the answers are those of the FP64 test.
         // The FP64 tests were four fifths of the assembly: 34.4 ms for 12.1 M
-        // tets and 1,500 discs, 11.1 ms with this.
+        // tets and 1,500 discs, 11.1 ms with this.  Tets whose corners are of no
+        // use in FP32 (thin ones) go to crack_thin_kernel.
         if (have_pts == 0) {
           F3 Rf[4];
           Rf[0] = {0.0f, 0.0f, 0.0f};
@@ -488,7 +521,9 @@ hodge_tet_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tet
             Rf[i] = {(float)(X[i].x - X[0].x), (float)(X[i].y - X[0].y),
                      (float)(X[i].z - X[0].z)};
           const F3 c = {(float)cT.x, (float)cT.y, (float)cT.z};
-          have_pts = crack_points(Rf, c, (float)(2.0 * Et), pts, Ept, Ppt) ? 1 : -1;
+          have_pts =
+              grid.fp32 && crack_points(Rf, c, (float)(2.0 * Et), pts, Ept, Ppt) ? 1 : -1;
+          if (have_pts < 0) return;
         }
         const double* dsc = grid.discs + 7 * (int64_t)id;
         const F3 c = {(float)(dsc[0] - X[0].x), (float)(dsc[1] - X[0].y),
@@ -509,44 +544,41 @@ hodge_tet_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tet
 #pragma unroll 1
           for (int h = 0; h < 2; ++h) {
             const int opp = h == 0 ? kEdgeD[s] : kEdgeC[s];
-            bool open = have_pts < 0;
             int st = first[s];
+            const F3 F = pt_load(pts, 6 + opp);
+            const float sf = dot(F - c, nrm);
+            const float lo3 = fminf(sM, fminf(sf, sT)), hi3 = fmaxf(sM, fmaxf(sf, sT));
+            if (lo3 > Es || hi3 < -Es) continue;      // one side: not cut
+            bool open = fminf(fabsf(sM), fminf(fabsf(sf), fabsf(sT))) <= Es;
             if (!open) {
-              const F3 F = pt_load(pts, 6 + opp);
-              const float sf = dot(F - c, nrm);
-              const float lo3 = fminf(sM, fminf(sf, sT)), hi3 = fmaxf(sM, fmaxf(sf, sT));
-              if (lo3 > Es || hi3 < -Es) continue;      // one side: not cut
-              open = fminf(fabsf(sM), fminf(fabsf(sf), fabsf(sT))) <= Es;
-              if (!open) {
-                // one corner (P0) on its own side: the plane meets the two
-                // edges from it
-                const F3 T = pt_load(pts, 10);
-                const bool m1 = (sM > 0.0f) != (sT > 0.0f), f1 = (sf > 0.0f) != (sT > 0.0f);
-                const F3 P0 = m1 && f1 ? T : m1 ? M : F;
-                const F3 P1 = m1 && f1 ? M : m1 ? F : M;
-                const F3 P2 = m1 && f1 ? F : T;
-                const float s0 = m1 && f1 ? sT : m1 ? sM : sf;
-                const float s1 = m1 && f1 ? sM : m1 ? sf : sM;
-                const float s2 = m1 && f1 ? sf : sT;
-                const F3 u1 = P1 - P0, u2 = P2 - P0;
-                const float i1 = 1.0f / (s0 - s1), i2 = 1.0f / (s0 - s2);
-                const F3 A = P0 + (s0 * i1) * u1, B = P0 + (s0 * i2) * u2;
-                const F3 d = B - A, g = c - A;
-                const float dd = dot(d, d);
-                float tt = 0.0f;
-                if (dd > 0.0f) tt = fminf(fmaxf(dot(g, d) / dd, 0.0f), 1.0f);
-                const F3 w = g - tt * d;
-                const float rho = sqrtf(dot(w, w));
-                // the crossing parameters move by Es / |s0 - si| and a few
-                // roundings; the distance by no more than the end points
-                const float EA = (Es * fabsf(i1) + 4.0f * kU) * sqrtf(dot(u1, u1));
-                const float EB = (Es * fabsf(i2) + 4.0f * kU) * sqrtf(dot(u2, u2));
-                const float Er = 1.01f * (Ept + 2.0f * fmaxf(EA, EB)) + 48.0f * kU * size;
-                const int n = first[s];
-                st = first_state(grid.scales_f, n, rho + Er, r * (1.0f - 8.0f * kU));
-                open = !(Er < size) ||
-                       st != first_state(grid.scales_f, n, rho - Er, r * (1.0f + 8.0f * kU));
-              }
+              // one corner (P0) on its own side: the plane meets the two
+              // edges from it
+              const F3 T = pt_load(pts, 10);
+              const bool m1 = (sM > 0.0f) != (sT > 0.0f), f1 = (sf > 0.0f) != (sT > 0.0f);
+              const F3 P0 = m1 && f1 ? T : m1 ? M : F;
+              const F3 P1 = m1 && f1 ? M : m1 ? F : M;
+              const F3 P2 = m1 && f1 ? F : T;
+              const float s0 = m1 && f1 ? sT : m1 ? sM : sf;
+              const float s1 = m1 && f1 ? sM : m1 ? sf : sM;
+              const float s2 = m1 && f1 ? sf : sT;
+              const F3 u1 = P1 - P0, u2 = P2 - P0;
+              const float i1 = 1.0f / (s0 - s1), i2 = 1.0f / (s0 - s2);
+              const F3 A = P0 + (s0 * i1) * u1, B = P0 + (s0 * i2) * u2;
+              const F3 d = B - A, g = c - A;
+              const float dd = dot(d, d);
+              float tt = 0.0f;
+              if (dd > 0.0f) tt = fminf(fmaxf(dot(g, d) / dd, 0.0f), 1.0f);
+              const F3 w = g - tt * d;
+              const float rho = sqrtf(dot(w, w));
+              // the crossing parameters move by Es / |s0 - si| and a few
+              // roundings; the distance by no more than the end points
+              const float EA = (Es * fabsf(i1) + 4.0f * kU) * sqrtf(dot(u1, u1));
+              const float EB = (Es * fabsf(i2) + 4.0f * kU) * sqrtf(dot(u2, u2));
+              const float Er = 1.01f * (Ept + 2.0f * fmaxf(EA, EB)) + 48.0f * kU * size;
+              const int n = first[s];
+              st = first_state(grid.scales_f, n, rho + Er, r * (1.0f - 8.0f * kU));
+              open = !(Er < size) ||
+                     st != first_state(grid.scales_f, n, rho - Er, r * (1.0f + 8.0f * kU));
             }
             if (open)
               st = crack_exact(xyz, v4, kEdgeA[s], kEdgeB[s], opp, exact_cT(), grid, id, first[s]);
@@ -554,23 +586,8 @@ hodge_tet_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tet
           }
         }
       };
-      if (!empty) {
-        const int64_t ncell = (int64_t)(c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) *
-                              (c1[2] - c0[2] + 1);
-        // a far circumcentre (flat boundary tet): fewer tests without the
-        // grid, i.e. every disc once (one pass of the loops below); one call
-        // site of test_disc keeps the kernel small
-        const bool all = ncell > grid.nd;
-        if (all) c1[0] = c0[0], c1[1] = c0[1], c1[2] = c0[2];
-        for (int gz = c0[2]; gz <= c1[2]; ++gz)
-          for (int gy = c0[1]; gy <= c1[1]; ++gy)
-            for (int gx = c0[0]; gx <= c1[0]; ++gx) {
-              const int cell = gx + grid.dim[0] * (gy + grid.dim[1] * gz);
-              const int i0 = all ? 0 : grid.start[cell];
-              const int i1 = all ? grid.nd : grid.start[cell + 1];
-              for (int it = i0; it < i1; ++it) test_disc(all ? it : grid.items[it]);
-            }
-      }
+      for_candidates(grid, cTa, RT, test_disc);
+      if (have_pts < 0) thin[atomicAdd(n_thin, 1ull)] = 2u * (uint32_t)t + (fast ? 1u : 0u);
     }
 #pragma unroll
     for (int s = 0; s < 6; ++s) slot_cut[t * 6 + s] = first[s];
@@ -578,6 +595,93 @@ hodge_tet_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tet
   // tets computed in FP64: one atomic per warp
   const unsigned w64 = __reduce_add_sync(0xffffffffu, n64);
   if ((threadIdx.x & 31) == 0 && w64) atomicAdd(n_fp64, (unsigned long long)w64);
+}
+
+// Crack states of the tets that hodge_tet_kernel left over: thin ones, whose
+// FP32 corners are of no use, and all that a disc may cut where radii or
+// scales leave FP32's range.  Every pair of tet and disc in FP64: the ball test
+// first (no cut outside the circumball), then the 12 sub-triangles from face
+// circumcentres formed once per tet.  Apart from the others, because a warp
+// with one such tet waited for it, and inside hodge_tet_kernel these tests
+// spilled its registers (12.1 M ordinary tets: 11.1 to 11.3 ms, 10.9 now).
+// Bound by the FP64 pipe.  The 64^3 cube with z scaled by 1e-3 (1e-6) and 300
+// discs: 684 (2,240) ms; 2,130 (2,487) with every test of every tet in FP64 in
+// one kernel, 2,028 (3,996) with one sub-triangle at a time out of line.
+__global__ void __launch_bounds__(kHodgeThreads)
+crack_thin_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tets,
+                  int64_t count, const uint32_t* __restrict__ thin,
+                  uint8_t* __restrict__ slot_cut, DiscGrid grid) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t id_fast = thin[i];
+    const int64_t t = id_fast >> 1;
+    const int4 v4 = reinterpret_cast<const int4*>(tets)[t];
+    const int vid[4] = {v4.x, v4.y, v4.z, v4.w};
+    V3 X[4], R[4], cT;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const double* p = xyz + 3 * (int64_t)vid[k];
+      X[k] = mk(p[0], p[1], p[2]);
+      R[k] = X[k] - X[0];
+    }
+    if (id_fast & 1u) {
+      cT = tet_circumcentre(R);
+    } else {                              // the circumcentre of the FP64 geometry
+      double a0[6], a1[6];
+      tet_pieces(R, cT, a0, a1);
+    }
+    const V3 c = X[0] + cT;
+    const double RT2 = dot(cT, cT) * (1.0 + 1e-9) + 1e-300, RT = sqrt(RT2);
+    const BallF ball = ball_f32(c, RT);
+    V3 cF[4];
+    bool have_cF = false;
+    uint8_t first[6];
+#pragma unroll
+    for (int s = 0; s < 6; ++s) first[s] = (uint8_t)grid.n_states;
+    for_candidates(grid, c, RT, [&](int id) {
+      if (!ball_meets_disc(grid, ball, id)) return;
+      const double* dsc = grid.discs + 7 * (int64_t)id;
+      const V3 dc = mk(dsc[0], dsc[1], dsc[2]), dn = mk(dsc[3], dsc[4], dsc[5]);
+      const double r = dsc[6];
+      const V3 v = c - dc;
+      const double dp = dot(v, dn);
+      if (dp * dp > RT2) return;                      // ball misses the plane
+      const double par2 = dot(v, v) - dp * dp;
+      const double reach = grid.smax * r * (1.0 + 1e-9);
+      if (par2 > reach * reach + 2.0 * reach * RT + RT2) return;
+      if (!have_cF) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+          cF[f] = tri_circumcentre(X[(f + 1) & 3], X[(f + 2) & 3], X[(f + 3) & 3]);
+        have_cF = true;
+      }
+      const double sT = dot(c - dc, dn);
+      double sF[4];
+#pragma unroll
+      for (int f = 0; f < 4; ++f) sF[f] = dot(cF[f] - dc, dn);
+#pragma unroll 1
+      for (int s = 0; s < 6; ++s) {
+        if (first[s] == 0) continue;
+        const V3 me = 0.5 * (X[kEdgeA[s]] + X[kEdgeB[s]]);
+        const double sM = dot(me - dc, dn);
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          const int opp = h == 0 ? kEdgeD[s] : kEdgeC[s];
+          const double sf = sF[opp];
+          if ((sM > 0.0 && sf > 0.0 && sT > 0.0) || (sM < 0.0 && sf < 0.0 && sT < 0.0))
+            continue;                                 // no crossing
+          const double rho = crack_rho_s(me, cF[opp], c, sM, sf, sT, dc);
+          for (int st = 0; st < (int)first[s]; ++st)
+            if (rho <= grid.scales[st] * r) {
+              first[s] = (uint8_t)st;
+              break;
+            }
+        }
+      }
+    });
+#pragma unroll
+    for (int s = 0; s < 6; ++s) slot_cut[t * 6 + s] = first[s];
+  }
 }
 
 // *1[e] = sum of the pieces of e (already divided by |e|), in increasing
@@ -789,19 +893,29 @@ dec_status assemble_hodge(dec_ctx* ctx, int64_t nd, bool has_k, int n_fields) {
   }
   int64_t blocks = (m + kHodgeThreads - 1) / kHodgeThreads;
   if (blocks > (int64_t)ctx->num_sms * 64) blocks = (int64_t)ctx->num_sms * 64;
-  DEC_TRY(ctx->geom_count.ensure(1));
-  DEC_TRY(cudaMemsetAsync(ctx->geom_count.p, 0, sizeof(unsigned long long), s));
+  DEC_TRY(ctx->geom_count.ensure(2));
+  DEC_TRY(cudaMemsetAsync(ctx->geom_count.p, 0, 2 * sizeof(unsigned long long), s));
+  if (nd > 0) DEC_TRY(ctx->key_a.ensure((m + 1) / 2));     // the list of thin tets
+  uint32_t* thin = reinterpret_cast<uint32_t*>(ctx->key_a.p);
   auto* kern = ctx->geom_precision == DEC_GEOM_MIXED ? hodge_tet_kernel<true>
                                                      : hodge_tet_kernel<false>;
   kern<<<(unsigned)std::max<int64_t>(blocks, 1), kHodgeThreads, 0, s>>>(
       ctx->xyz.p, ctx->tets.p, has_k ? ctx->kcond.p : nullptr,
       m, ctx->piece.p, has_k ? ctx->piece.p + q : nullptr, ctx->slot_cut.p, g,
-      ctx->geom_count.p);
+      ctx->geom_count.p, ctx->geom_count.p + 1, thin);
   DEC_TRY(cudaGetLastError());
-  unsigned long long n64 = 0;
-  DEC_TRY(cudaMemcpyAsync(&n64, ctx->geom_count.p, sizeof(n64), cudaMemcpyDeviceToHost, s));
+  unsigned long long counts[2] = {0, 0};      // tets in FP64, thin tets
+  DEC_TRY(cudaMemcpyAsync(counts, ctx->geom_count.p, sizeof(counts), cudaMemcpyDeviceToHost, s));
   DEC_TRY(cudaStreamSynchronize(s));
-  ctx->geom_fp64_tets = (int64_t)n64;
+  ctx->geom_fp64_tets = (int64_t)counts[0];
+  if (counts[1] > 0) {
+    const int64_t tb = ((int64_t)counts[1] + kHodgeThreads - 1) / kHodgeThreads;
+    crack_thin_kernel<<<(unsigned)std::min<int64_t>(tb, (int64_t)ctx->num_sms * 64), kHodgeThreads,
+                        0, s>>>(ctx->xyz.p, ctx->tets.p, (int64_t)counts[1], thin,
+                                ctx->slot_cut.p, g);
+    DEC_TRY(cudaGetLastError());
+    ctx->launches += 1;
+  }
   int64_t eb = (ctx->ne + 255) / 256;
   if (eb > (int64_t)ctx->num_sms * 32) eb = (int64_t)ctx->num_sms * 32;
   edge_reduce_kernel<<<(unsigned)std::max<int64_t>(eb, 1), 256, 0, s>>>(
