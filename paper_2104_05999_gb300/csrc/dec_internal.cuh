@@ -394,6 +394,9 @@ dec_status radix_sort_pairs(dec_ctx* ctx, uint64_t* keys, uint32_t* vals,
                             int key_bits, bool* result_in_alt);
 // mesh
 dec_status build_mesh(dec_ctx* ctx, bool* radix);
+// the rows of nodes with many lower neighbours, which build_mesh leaves open
+// (errflag bit 256)
+dec_status build_hub_rows(dec_ctx* ctx);
 dec_status build_edges(dec_ctx* ctx);
 dec_status build_csr_structure(dec_ctx* ctx);
 dec_status build_sell_layouts(dec_ctx* ctx, int* flags);

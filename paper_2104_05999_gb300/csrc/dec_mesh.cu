@@ -9,8 +9,9 @@
 // writes every entry three times.  Sorting (64-bit key, payload) pairs of the
 // whole mesh by radix took six passes of 32 bytes per entry; with the row
 // structure built the same way, an upload of 2.05 M nodes (12.1 M tets) went
-// from 14.6 to 4.7 ms.  The radix path stays for meshes with a node of more
-// than kGroupMax entries, which one warp would sort too slowly.
+// from 14.6 to 4.7 ms.  Nodes of more than kWarpMax entries or lower
+// neighbours (hubs) get a block each, in launches that other meshes do not
+// make; the radix path stays for meshes with a node of more than kGroupMax.
 #include "dec_internal.cuh"
 
 #include <algorithm>
@@ -22,7 +23,7 @@ __constant__ int kLocalEdge[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2,
 // ----------------------------------------------------------- validation
 // errflag bit 1: node id out of range, bit 2: tet not positively oriented,
 // bit 4: bad node tag; 32, 64: a node's edges or lower neighbours are too
-// many for the grouped sorts.
+// many for the grouped sorts; 128, 256: too many for a warp.
 
 // FP32 value of a double, truncated by integer operations (conversions run on
 // the narrow FP64 pipe); infinity stands for anything out of FP32's range.
@@ -125,6 +126,12 @@ __global__ void tet_count_kernel(const int32_t* __restrict__ tets,
 
 // -------------------------------------------- edges grouped by smaller node
 constexpr int kGroupMax = 4096;   // entries (or lower neighbours) of one node
+// As many are ranked by one warp (lower neighbours: by eight lanes), in
+// n^2 / 32 (n^2 / 8) steps; a block sorts more.  Uploads of 60 spheres of tets
+// around a hub, ms with warps alone / with blocks / with radix sorts: hub of
+// 252 entries .26 / - / .48, 486 .40 / .25 / .54, 1,014 1.0 / .30 / .57, 4,056
+// 12.8 / .53 / .70; of 326 lower neighbours .40 / .25 / .65, 3,846 21.7 / .74 / 2.6.
+constexpr int kWarpMax = 256;
 
 // local edge slot of the local vertex pair {a, b}: (0,1) (0,2) (0,3) (1,2)
 // (1,3) (2,3)
@@ -172,8 +179,8 @@ group_sort_kernel(int64_t n, const uint32_t* __restrict__ beg, const uint64_t* _
     const uint32_t b0 = beg[i];
     const int c = (int)(beg[i + 1] - b0);
     int heads = 0;
-    if (c > kGroupMax) {
-      if (lane == 0) atomicOr(errflag, 32);
+    if (c > kWarpMax) {
+      if (lane == 0) atomicOr(errflag, c > kGroupMax ? 32 : 128);
     } else if (c <= kGroupSmem) {
       const uint64_t none = ~0ull;
       const uint64_t k0 = lane < c ? in[b0 + lane] : none;
@@ -219,6 +226,66 @@ group_sort_kernel(int64_t n, const uint32_t* __restrict__ beg, const uint64_t* _
     }
     if (lane == 0) ucnt[i] = (uint32_t)heads;
   }
+}
+
+// Sort the c <= kGroupMax keys in `key` (bitonic network, all threads)
+constexpr int kHubBlock = 1024;
+__device__ __forceinline__ void block_sort(uint64_t* key, int c) {
+  int P = 2;
+  while (P < c) P <<= 1;
+  for (int i = c + threadIdx.x; i < P; i += kHubBlock) key[i] = ~0ull;
+  __syncthreads();
+  for (int k = 2; k <= P; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int h = threadIdx.x; h < P / 2; h += kHubBlock) {
+        const int a = 2 * h - (h & (j - 1)), b = a + j;
+        const uint64_t x = key[a], y = key[b];
+        if ((x > y) == ((a & k) == 0)) {
+          key[a] = y;
+          key[b] = x;
+        }
+      }
+      __syncthreads();
+    }
+}
+
+// body(node, size) by a whole block for every node of more than kWarpMax
+// items (begin[i + 1] - begin[i]); 32 nodes are looked at a time
+template <typename T, typename Body>
+__device__ __forceinline__ void for_hubs(int64_t n, const T* __restrict__ begin, Body&& body) {
+  __shared__ int size[32];
+  for (int64_t i0 = blockIdx.x * (int64_t)32; i0 < n; i0 += gridDim.x * (int64_t)32) {
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const int64_t i = i0 + threadIdx.x;
+      const int c = i < n ? (int)(begin[i + 1] - begin[i]) : 0;
+      size[threadIdx.x] = c > kWarpMax && c <= kGroupMax ? c : 0;
+    }
+    __syncthreads();
+    for (int h = 0; h < 32; ++h)
+      if (size[h]) body(i0 + h, size[h]);
+  }
+}
+
+// group_sort_kernel's work for hubs
+__global__ void __launch_bounds__(kHubBlock)
+group_sort_hubs_kernel(int64_t n, const uint32_t* __restrict__ beg,
+                       const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
+                       uint32_t* __restrict__ ucnt) {
+  __shared__ uint64_t key[kGroupMax];
+  for_hubs(n, beg, [&](int64_t i, int c) {
+    const uint32_t b0 = beg[i];
+    for (int e = threadIdx.x; e < c; e += kHubBlock) key[e] = in[b0 + e];
+    block_sort(key, c);
+    int heads = 0;
+    for (int e0 = 0; e0 < c; e0 += kHubBlock) {
+      const int e = e0 + threadIdx.x;
+      if (e < c) out[b0 + e] = key[e];
+      heads += __syncthreads_count(e < c && (e == 0 || (key[e - 1] >> 32) != (key[e] >> 32)));
+    }
+    if (threadIdx.x == 0) ucnt[i] = (uint32_t)heads;
+    __syncthreads();
+  });
 }
 
 // One warp per node: edge ids of its sorted entries (edges are numbered by
@@ -284,8 +351,8 @@ csr_rows_kernel(int64_t n, const int32_t* __restrict__ E, const int32_t* __restr
                 const int32_t* __restrict__ lo, const uint32_t* __restrict__ list,
                 int32_t* __restrict__ rowptr, int32_t* __restrict__ col,
                 int32_t* __restrict__ eid, int32_t* __restrict__ dpos,
-                int32_t* __restrict__ pos_up, const int* __restrict__ errflag) {
-  if (*errflag & 64) return;                // the radix path takes over
+                int32_t* __restrict__ pos_up, int* errflag) {
+  if (*(volatile int*)errflag & 64) return;   // the radix path takes over
   const int lane = threadIdx.x & 7;
   for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3; r <= n;
        r += ((int64_t)gridDim.x * blockDim.x) >> 3) {
@@ -294,7 +361,8 @@ csr_rows_kernel(int64_t n, const int32_t* __restrict__ E, const int32_t* __restr
     if (lane == 0) rowptr[r] = p0;
     if (r == n) break;
     const int32_t nl = lo[r + 1] - l0, nu = up[r + 1] - u0;
-    for (int32_t k = lane; k < nl; k += 8) {
+    if (nl > kWarpMax && lane == 0) atomicOr(errflag, 256);    // csr_hub_rows_kernel
+    for (int32_t k = lane; k < nl && nl <= kWarpMax; k += 8) {
       const uint32_t e = list[l0 + k];
       int32_t rank = 0;
       for (int32_t j = 0; j < nl; ++j) rank += list[l0 + j] < e;
@@ -314,6 +382,25 @@ csr_rows_kernel(int64_t n, const int32_t* __restrict__ E, const int32_t* __restr
       pos_up[e] = pd + 1 + k;
     }
   }
+}
+
+// The lower neighbours of hubs in csr_rows_kernel's rows
+__global__ void __launch_bounds__(kHubBlock)
+csr_hub_rows_kernel(int64_t n, const int32_t* __restrict__ E, const int32_t* __restrict__ lo,
+                    const uint32_t* __restrict__ list, const int32_t* __restrict__ rowptr,
+                    int32_t* __restrict__ col, int32_t* __restrict__ eid) {
+  __shared__ uint64_t key[kGroupMax];
+  for_hubs(n, lo, [&](int64_t r, int nl) {
+    const int32_t l0 = lo[r], p0 = rowptr[r];
+    for (int k = threadIdx.x; k < nl; k += kHubBlock) key[k] = list[l0 + k];
+    block_sort(key, nl);
+    for (int k = threadIdx.x; k < nl; k += kHubBlock) {
+      const int32_t e = (int32_t)key[k];
+      col[p0 + k] = E[2 * (int64_t)e];
+      eid[p0 + k] = e;
+    }
+    __syncthreads();
+  });
 }
 
 // ------------------------------------------------------------ edge list
@@ -540,6 +627,18 @@ static dec_status mesh_errors(dec_ctx* ctx, int flag) {
   return DEC_OK;
 }
 
+static unsigned hub_grid(const dec_ctx* ctx) {
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>((ctx->n + 31) / 32, ctx->num_sms * 2));
+}
+
+dec_status build_hub_rows(dec_ctx* ctx) {
+  csr_hub_rows_kernel<<<hub_grid(ctx), kHubBlock, 0, ctx->stream>>>(
+      ctx->n, ctx->E.p, ctx->lo_begin.p, ctx->val_b.p, ctx->rowptr.p, ctx->col.p, ctx->eid.p);
+  DEC_TRY(cudaGetLastError());
+  ctx->launches += 1;
+  return DEC_OK;
+}
+
 // Mesh checks, edge list and CSR structure.  *radix is set when a node has
 // more than kGroupMax edges or lower neighbours: the first is known here and
 // nothing but the checks has been done, the second only once the caller reads
@@ -584,6 +683,18 @@ dec_status build_mesh(dec_ctx* ctx, bool* radix) {
   if (flag & 32) {
     *radix = true;
     return DEC_OK;
+  }
+  if (flag & 128) {      // hubs: counted again with the others, whose counts are summed by now
+    group_sort_kernel<<<gn, 32 * kGroupWarps, 0, s>>>(n, beg, ctx->key_a.p, ctx->key_b.p, up,
+                                                      ctx->errflag.p);
+    group_sort_hubs_kernel<<<hub_grid(ctx), kHubBlock, 0, s>>>(n, beg, ctx->key_a.p, ctx->key_b.p,
+                                                               up);
+    DEC_TRY(cudaGetLastError());
+    DEC_TRY(cudaMemsetAsync(up + n, 0, sizeof(uint32_t), s));
+    DEC_TRY(exclusive_scan_u32(up, up, n + 1, ctx->scan_tmp.p, ctx->scan_tmp.cap, s));
+    DEC_TRY(cudaMemcpyAsync(&ne, up + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    DEC_TRY(cudaStreamSynchronize(s));
+    ctx->launches += 2 + 3;
   }
   ctx->ne = ne;
   ctx->nnz = 2 * ctx->ne + n;

@@ -267,6 +267,7 @@ dec_status build_sell_layouts(dec_ctx* ctx, int* flags) {
   DEC_TRY(cudaStreamSynchronize(s));
   ctx->launches += 5;
   if (*flags & 64) return DEC_OK;
+  if (*flags & 256) DEC_TRY_STATUS(build_hub_rows(ctx));
   uint32_t before = 0;
   for (int k = 0; k < 3; ++k) {
     M[k]->total = (uint32_t)(end[k] - before);   // a matrix has fewer than 2^32 entries
