@@ -138,7 +138,7 @@ dec_status dec_mesh_upload(dec_ctx* ctx, const double* xyz, int64_t n_nodes,
   int flags = 0;
   DEC_TRY_STATUS(dec::build_mesh(ctx, &radix));
   if (!radix) DEC_TRY_STATUS(dec::build_sell_layouts(ctx, &flags));
-  if (radix || (flags & 64)) {     // a node with thousands of edges
+  if (radix || (flags & 64)) {     // a node with more edges than a block sorts
     DEC_TRY(cudaMemsetAsync(ctx->errflag.p, 0, sizeof(int), s));
     DEC_TRY_STATUS(dec::build_edges(ctx));
     DEC_TRY_STATUS(dec::build_csr_structure(ctx));

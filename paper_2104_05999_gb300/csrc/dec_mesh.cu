@@ -125,7 +125,10 @@ __global__ void tet_count_kernel(const int32_t* __restrict__ tets,
 }
 
 // -------------------------------------------- edges grouped by smaller node
-constexpr int kGroupMax = 4096;   // entries (or lower neighbours) of one node
+// Entries (or lower neighbours) of one node: what a block sorts in 128 KB of
+// shared memory.  A mesh with a larger node is found out late, after 0.5 to 0.8
+// of 7 ms at 5.9 M tets, and sorted by radix.
+constexpr int kGroupMax = 16384;
 // As many are ranked by one warp (lower neighbours: by eight lanes), in
 // n^2 / 32 (n^2 / 8) steps; a block sorts more.  Uploads of 60 spheres of tets
 // around a hub, ms with warps alone / with blocks / with radix sorts: hub of
@@ -272,7 +275,7 @@ __global__ void __launch_bounds__(kHubBlock)
 group_sort_hubs_kernel(int64_t n, const uint32_t* __restrict__ beg,
                        const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
                        uint32_t* __restrict__ ucnt) {
-  __shared__ uint64_t key[kGroupMax];
+  extern __shared__ uint64_t key[];
   for_hubs(n, beg, [&](int64_t i, int c) {
     const uint32_t b0 = beg[i];
     for (int e = threadIdx.x; e < c; e += kHubBlock) key[e] = in[b0 + e];
@@ -389,7 +392,7 @@ __global__ void __launch_bounds__(kHubBlock)
 csr_hub_rows_kernel(int64_t n, const int32_t* __restrict__ E, const int32_t* __restrict__ lo,
                     const uint32_t* __restrict__ list, const int32_t* __restrict__ rowptr,
                     int32_t* __restrict__ col, int32_t* __restrict__ eid) {
-  __shared__ uint64_t key[kGroupMax];
+  extern __shared__ uint64_t key[];
   for_hubs(n, lo, [&](int64_t r, int nl) {
     const int32_t l0 = lo[r], p0 = rowptr[r];
     for (int k = threadIdx.x; k < nl; k += kHubBlock) key[k] = list[l0 + k];
@@ -628,11 +631,14 @@ static dec_status mesh_errors(dec_ctx* ctx, int flag) {
 }
 
 static unsigned hub_grid(const dec_ctx* ctx) {
-  return (unsigned)std::max<int64_t>(1, std::min<int64_t>((ctx->n + 31) / 32, ctx->num_sms * 2));
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>((ctx->n + 31) / 32, ctx->num_sms));
 }
 
 dec_status build_hub_rows(dec_ctx* ctx) {
-  csr_hub_rows_kernel<<<hub_grid(ctx), kHubBlock, 0, ctx->stream>>>(
+  constexpr int smem = kGroupMax * sizeof(uint64_t);
+  DEC_TRY(cudaFuncSetAttribute(csr_hub_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               smem));
+  csr_hub_rows_kernel<<<hub_grid(ctx), kHubBlock, smem, ctx->stream>>>(
       ctx->n, ctx->E.p, ctx->lo_begin.p, ctx->val_b.p, ctx->rowptr.p, ctx->col.p, ctx->eid.p);
   DEC_TRY(cudaGetLastError());
   ctx->launches += 1;
@@ -687,8 +693,11 @@ dec_status build_mesh(dec_ctx* ctx, bool* radix) {
   if (flag & 128) {      // hubs: counted again with the others, whose counts are summed by now
     group_sort_kernel<<<gn, 32 * kGroupWarps, 0, s>>>(n, beg, ctx->key_a.p, ctx->key_b.p, up,
                                                       ctx->errflag.p);
-    group_sort_hubs_kernel<<<hub_grid(ctx), kHubBlock, 0, s>>>(n, beg, ctx->key_a.p, ctx->key_b.p,
-                                                               up);
+    constexpr int smem = kGroupMax * sizeof(uint64_t);
+    DEC_TRY(cudaFuncSetAttribute(group_sort_hubs_kernel,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    group_sort_hubs_kernel<<<hub_grid(ctx), kHubBlock, smem, s>>>(n, beg, ctx->key_a.p,
+                                                                  ctx->key_b.p, up);
     DEC_TRY(cudaGetLastError());
     DEC_TRY(cudaMemsetAsync(up + n, 0, sizeof(uint32_t), s));
     DEC_TRY(exclusive_scan_u32(up, up, n + 1, ctx->scan_tmp.p, ctx->scan_tmp.cap, s));
