@@ -1546,7 +1546,7 @@ static dec_status build_morton(dec_ctx* ctx) {
   morton_keys_kernel<<<grid_for_work(ctx, n), 256, 0, s>>>(n, ctx->xyz.p, lo, sc, t,
                                                            ctx->key_a.p, ctx->val_a.p);
   DEC_TRY(cudaGetLastError());
-  ctx->launches += 2;
+  ctx->launches += 3;
   bool alt = false;
   DEC_TRY_STATUS(radix_sort_pairs(ctx, ctx->key_a.p, ctx->val_a.p, ctx->key_b.p, ctx->val_b.p,
                                   n, 63, &alt));

@@ -889,7 +889,7 @@ dec_status assemble_hodge(dec_ctx* ctx, int64_t nd, bool has_k, int n_fields) {
     DEC_TRY(cudaGetLastError());
     g.start = counts;
     g.items = ctx->grid_items.p;
-    ctx->launches += 6;  // count, scan (3), cursor copy, fill
+    ctx->launches += 3 + scan_launches(cells + 1);  // count, cursor copy, fill
   }
   int64_t blocks = (m + kHodgeThreads - 1) / kHodgeThreads;
   if (blocks > (int64_t)ctx->num_sms * 64) blocks = (int64_t)ctx->num_sms * 64;

@@ -389,6 +389,7 @@ namespace dec {
 cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n,
                                uint32_t* tmp, size_t tmp_cap, cudaStream_t s);
 size_t scan_tmp_size(int64_t n);
+int scan_launches(int64_t n);
 dec_status radix_sort_pairs(dec_ctx* ctx, uint64_t* keys, uint32_t* vals,
                             uint64_t* keys_alt, uint32_t* vals_alt, int64_t n,
                             int key_bits, bool* result_in_alt);

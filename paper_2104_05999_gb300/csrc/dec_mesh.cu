@@ -481,7 +481,7 @@ dec_status build_edges(dec_ctx* ctx) {
   edge_keys_kernel<<<grid_for(ctx, ctx->m, 256), 256, 0, s>>>(
       ctx->tets.p, ctx->m, n, ctx->key_a.p, ctx->val_a.p);
   DEC_TRY(cudaGetLastError());
-  ctx->launches += 1 + 1 + 3 + 1;  // keys, heads, scan, emit (sort counts itself)
+  ctx->launches += 3 + scan_launches(q);  // keys, heads, emit (the sort counts itself)
   bool alt = false;
   DEC_TRY_STATUS(radix_sort_pairs(ctx, ctx->key_a.p, ctx->val_a.p, ctx->key_b.p,
                                   ctx->val_b.p, q, key_bits_for(n), &alt));
@@ -679,7 +679,7 @@ dec_status build_mesh(dec_ctx* ctx, bool* radix) {
   DEC_TRY(cudaGetLastError());
   DEC_TRY(cudaMemsetAsync(up + n, 0, sizeof(uint32_t), s));
   DEC_TRY(exclusive_scan_u32(up, up, n + 1, ctx->scan_tmp.p, ctx->scan_tmp.cap, s));
-  ctx->launches += 3 + 6;
+  ctx->launches += 3 + 2 * scan_launches(n + 1);
   int flag = 0;
   uint32_t ne = 0;
   DEC_TRY(cudaMemcpyAsync(&flag, ctx->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -703,7 +703,7 @@ dec_status build_mesh(dec_ctx* ctx, bool* radix) {
     DEC_TRY(exclusive_scan_u32(up, up, n + 1, ctx->scan_tmp.p, ctx->scan_tmp.cap, s));
     DEC_TRY(cudaMemcpyAsync(&ne, up + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     DEC_TRY(cudaStreamSynchronize(s));
-    ctx->launches += 2 + 3;
+    ctx->launches += 2 + scan_launches(n + 1);
   }
   ctx->ne = ne;
   ctx->nnz = 2 * ctx->ne + n;
@@ -732,7 +732,7 @@ dec_status build_mesh(dec_ctx* ctx, bool* radix) {
       n, ctx->E.p, ctx->up_begin.p, ctx->lo_begin.p, ctx->val_b.p, ctx->rowptr.p, ctx->col.p,
       ctx->eid.p, ctx->dpos.p, ctx->pos_up.p, ctx->errflag.p);
   DEC_TRY(cudaGetLastError());
-  ctx->launches += 3 + 3;
+  ctx->launches += 3 + scan_launches(n + 1);
   return DEC_OK;
 }
 

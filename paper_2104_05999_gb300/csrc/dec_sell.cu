@@ -155,7 +155,7 @@ dec_status build_sell(dec_ctx* ctx, int kind, SellLayout& L, int C, int R,
       kind, L.nslices, C, ctx->rowptr.p, ctx->dpos.p, ctx->col.p, ctx->tag.p, L.perm.p,
       L.sptr.p, L.col.p, L.pos.p);
   DEC_TRY(cudaGetLastError());
-  ctx->launches += 6;  // sort, widths, scan (3), fill
+  ctx->launches += 3 + scan_launches(L.nslices + 1);  // sort, widths, fill
   return DEC_OK;
 }
 
@@ -265,7 +265,7 @@ dec_status build_sell_layouts(dec_ctx* ctx, int* flags) {
                             cudaMemcpyDeviceToHost, s));
   DEC_TRY(cudaMemcpyAsync(flags, ctx->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   DEC_TRY(cudaStreamSynchronize(s));
-  ctx->launches += 5;
+  ctx->launches += 2 + scan_launches(cnt);
   if (*flags & 64) return DEC_OK;
   if (*flags & 256) DEC_TRY_STATUS(build_hub_rows(ctx));
   uint32_t before = 0;

@@ -107,6 +107,11 @@ scan_down_kernel(const uint32_t* in, uint32_t* out,
 
 size_t scan_tmp_size(int64_t n) { return (size_t)((n + kScanTile - 1) / kScanTile) + 1; }
 
+constexpr int64_t kScanOneBlock = 8 * 1024;
+
+// kernels that exclusive_scan_u32 launches for n entries in place
+int scan_launches(int64_t n) { return n <= 0 ? 0 : n <= kScanOneBlock ? 1 : 3; }
+
 // out[i] = sum_{k < i} in[k]; in == out is allowed.  `tmp` needs
 // scan_tmp_size(n) entries.
 cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n,
@@ -114,7 +119,7 @@ cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n,
   if (n <= 0) return cudaSuccess;
   int64_t nb = (n + kScanTile - 1) / kScanTile;
   if ((size_t)nb > tmp_cap) return cudaErrorInvalidValue;
-  if (in == out && n <= 8 * 1024) {      // one block, one launch
+  if (in == out && n <= kScanOneBlock) {      // one block, one launch
     scan_top_kernel<<<1, 1024, 0, s>>>(out, n);
     return cudaGetLastError();
   }
@@ -224,7 +229,7 @@ dec_status radix_sort_pairs(dec_ctx* ctx, uint64_t* keys, uint32_t* vals,
   for (int p = 0; p < passes; ++p) {
     const int shift = 8 * p;
     radix_hist_kernel<<<tiles, kSortThreads, 0, ctx->stream>>>(ki, n, shift, ctx->hist.p, tiles);
-    ctx->launches += 5;  // histogram, 3-kernel scan, scatter
+    ctx->launches += 2 + scan_launches(hn);  // histogram, scatter
     DEC_TRY(exclusive_scan_u32(ctx->hist.p, ctx->hist.p, hn, ctx->scan_tmp.p,
                                ctx->scan_tmp.cap, ctx->stream));
     radix_scatter_kernel<<<tiles, kSortThreads, 0, ctx->stream>>>(

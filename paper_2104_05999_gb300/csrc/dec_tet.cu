@@ -707,7 +707,7 @@ dec_status tet_faces(dec_ctx* ctx) {
                                                  ctx->faces.p, ctx->fslot0.p, ctx->fslot1.p,
                                                  ctx->t2f.p);
   DEC_TRY(cudaGetLastError());
-  ctx->launches += 7;   // keys, heads, scan (3), fill (the sort counts itself)
+  ctx->launches += 3 + scan_launches(q);   // keys, heads, fill (the sort counts itself)
   ctx->nf = nf;
   return DEC_OK;
 }
