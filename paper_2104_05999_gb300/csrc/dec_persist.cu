@@ -124,19 +124,19 @@ __device__ __forceinline__ bool grid_sum(const T (&v)[NV], double (&tot)[NV],
 // the fly: sum_j a_j * (X[c_j] + coef * Y[c_j]).  Used to fuse the vector
 // update that produced the operand into the product that consumes it (the
 // owner of row c computes the same fmaf for its own entry, so both agree).
-template <typename MT, typename VT>
-__device__ __forceinline__ VT sell_row2(const SellArg<MT>& A, int64_t s, int lane, const VT* X,
-                                        const VT* Y, VT coef) {
+template <typename MT>
+__device__ __forceinline__ float sell_row2(const SellArg<MT>& A, int64_t s, int lane,
+                                           const float* X, const float* Y, float coef) {
   constexpr int U = 8;
   const int32_t base = __ldg(A.sptr + s);
   const int32_t w = (__ldg(A.sptr + s + 1) - base) >> 5;
   const int32_t* __restrict__ cp = A.col + base + lane;
   const MT* __restrict__ vp = A.val + base + lane;
-  VT acc = VT(0);
+  float acc = 0.0f;
   for (int32_t j = 0; j < w; j += U) {
     int32_t c[U];
     MT av[U];
-    VT xv[U], yv[U];
+    float xv[U], yv[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const bool ok = j + u < w;
@@ -145,12 +145,12 @@ __device__ __forceinline__ VT sell_row2(const SellArg<MT>& A, int64_t s, int lan
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      xv[u] = j + u < w ? X[c[u]] : VT(0);
-      yv[u] = j + u < w ? Y[c[u]] : VT(0);
+      xv[u] = j + u < w ? X[c[u]] : 0.0f;
+      yv[u] = j + u < w ? Y[c[u]] : 0.0f;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (j + u < w) acc = fma_(av[u], fma_(coef, yv[u], xv[u]), acc);
+      if (j + u < w) acc = fma_(av[u], fmaf(coef, yv[u], xv[u]), acc);
   }
   return acc;
 }
