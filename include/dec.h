@@ -183,9 +183,10 @@ enum {
  * edge from its first vertex, V its volume; a regular tet has
  * L^3 / |6 V| = 2.8, a Kuhn tet 5.2) and L lies in [1e-7, 1e7], in FP64
  * otherwise.  Crack decisions
- * are those of the FP64 geometry: the FP32 circumcentre only serves as a
- * filter with an error bound, and any tet that a disc may cut has its
- * circumcentre formed again in FP64 for the exact test.  The FP32 pieces
+ * are those of the FP64 geometry with either choice: where a disc may cut a
+ * tet, signs and distances are decided in FP32 outside bounds on their errors
+ * (the circumcentre's among them) and in FP64, from the nodes, where a bound
+ * leaves one open.  The FP32 pieces
  * carry relative errors of order 1e-6, so *1, T and k_eff move by about
  * that much against the FP64 geometry (DEC_GEOM_FP64 keeps agreement with
  * the FP64 definition to 1e-12).  dec_get_geom_fp64_tets gives the number

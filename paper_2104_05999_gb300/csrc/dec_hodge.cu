@@ -601,9 +601,9 @@ hodge_tet_kernel(const double* __restrict__ xyz, const int32_t* __restrict__ tet
 // FP32 corners are of no use, and all that a disc may cut where radii or
 // scales leave FP32's range.  Every pair of tet and disc in FP64: the ball test
 // first (no cut outside the circumball), then the 12 sub-triangles from face
-// circumcentres formed once per tet.  Apart from the others, because a warp
-// with one such tet waited for it, and inside hodge_tet_kernel these tests
-// spilled its registers (12.1 M ordinary tets: 11.1 to 11.3 ms, 10.9 now).
+// circumcentres formed once per tet.  Apart from the others, because inside
+// hodge_tet_kernel these tests cost it registers (12.1 M ordinary tets: 11.1 to
+// 11.3 ms, 10.9 now).
 // Bound by the FP64 pipe.  The 64^3 cube with z scaled by 1e-3 (1e-6) and 300
 // discs: 684 (2,240) ms; 2,130 (2,487) with every test of every tet in FP64 in
 // one kernel, 2,028 (3,996) with one sub-triangle at a time out of line.

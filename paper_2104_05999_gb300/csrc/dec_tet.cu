@@ -480,10 +480,10 @@ __device__ __noinline__ double tet_product(const int4* __restrict__ col, int64_t
 // a true one that has not restarts from the true residual.  With FSAI the
 // preconditioned residual z lives in q between the update and p = z + beta p.
 // Five phases per iteration, between grid barriers, 280 B and 21 FMAs a row.
-// Bound by DRAM (103 us an iteration at 1.7 M rows: 4.6 TB/s if all of it
-// came from there) and, close behind, by the FP64 pipe (2 FMAs a clock and SM:
-// 57 us), so phases are not fused where a fused one would repeat an update
-// for every neighbour.  One block per SM: at 1,024 threads a quarter of the
+// 99 us an iteration at 1.7 M rows, no unit full (ncu): 342 of the 478 MB come
+// from DRAM (3.5 TB/s, 52 % of the copy rate), the FP64 pipe is 64 % busy, warps
+// wait for gathers and at barriers.  Phases are not fused where a fused one
+// would repeat an update for every neighbour on that pipe.  One block per SM: at 1,024 threads a quarter of the
 // partial sums, which every block adds up, of four blocks of 256.  The 64^3
 // cube's 1,084 iterations: 147 ms with slot-major rows, separate arrays for G
 // and G^T and four blocks of 256; 111 ms now.  More resident threads (1,536
