@@ -650,17 +650,15 @@ pcg_cluster_kernel(ClusterArgs a) {
     sum2(bb, 0.0, One{}, nothing);
   }
   const double bnorm2 = bc[0], tol2 = a.rtol2 * bnorm2;
-  double rr = bnorm2;
   // Only b = 0, or a warm start that meets the tolerance, needs no iteration;
-  // a right-hand side that is not finite breaks down in the first one.
-  bool solved = bnorm2 == 0.0;
-  if (a.warm && !solved) {
+  // the host reports a right-hand side that is not finite.
+  double rr = nan("");
+  if (a.warm && bnorm2 > 0.0) {
     residual();
     rr = bc[0];
-    solved = rr <= tol2 && isfinite(bnorm2);
   }
   int iters = 0, outcome = 0;
-  while (!solved) {
+  while (bnorm2 > 0.0 && !(rr <= tol2)) {
     // (re)start: z = M r, r.z, beta = 0
     double v = 0.0;
     const double* rc = a.r[cur];
@@ -748,14 +746,14 @@ pcg_cluster_kernel(ClusterArgs a) {
     // the true residual decides
     residual();
     rr = bc[0];
-    if (breakdown || !isfinite(bnorm2)) { outcome = 3; break; }
+    if (breakdown) { outcome = 3; break; }
     if (rr <= tol2) break;
     if (iters >= a.max_iter) { outcome = 1; break; }
   }
   if (rank == 0 && threadIdx.x == 0) {
     a.status[0] = iters;
     a.status[1] = outcome;
-    a.result[0] = bnorm2 == 0.0 ? 0.0 : rr;
+    a.result[0] = bnorm2 > 0.0 ? rr : 0.0;
     a.result[1] = bnorm2;
   }
   };
@@ -837,7 +835,8 @@ dec_status solve_fp64_cluster(dec_ctx* ctx, int inst, double rtol, int max_iter,
   memcpy(hr, h + 8, sizeof(hr));
   *iters_out = hs[0];
   *relres_out = hr[1] > 0.0 ? std::sqrt(hr[0] / hr[1]) : 0.0;
-  if (hs[1] == 3) return ctx->fail(DEC_ERR_BREAKDOWN, "CG breakdown: p.Lp <= 0 or not finite");
+  if (hs[1] == 3 || !std::isfinite(hr[1]))
+    return ctx->fail(DEC_ERR_BREAKDOWN, "CG breakdown: p.Lp <= 0 or not finite");
   if (hs[1] == 1) return ctx->fail(DEC_NOT_CONVERGED, "max_iter reached");
   return DEC_OK;
 }
