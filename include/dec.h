@@ -81,8 +81,9 @@ enum {
 /* solve modes (dec_solve) */
 enum {
   DEC_MODE_FP64 = 0,   /* PCG in FP64 (matrix, preconditioner, vectors): one
-                          launch per instance up to 6,000 nodes, one kernel
-                          per phase above                                  */
+                          launch per instance up to 6,000 nodes where the
+                          device can place a cluster of 16 blocks, one
+                          kernel per phase elsewhere                       */
   DEC_MODE_MIXED = 1,  /* PCG with FP32 vectors and L and a BF16 FSAI factor
                           (FP32 Jacobi) inside FP64 defect correction: the
                           FP32 update is added to an FP64 solution x and the

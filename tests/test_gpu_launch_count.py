@@ -36,7 +36,7 @@ def test_counted_launches_are_those_the_profiler_sees(N):
     with abi.Context(device=0) as ctx:
         ctx.dec_mesh_upload(wl.xyz, wl.tets, wl.tags)
         if not any(kernels(lambda: ctx.dec_hodge_assemble(None)) for _ in range(3)):
-            pytest.skip("no kernel records on this box")
+            pytest.skip("the profiler records no kernels here")
         steps = [lambda: ctx.dec_mesh_upload(hub_xyz, hub_tets,
                                              np.zeros(len(hub_xyz), dtype=np.uint8)),
                  lambda: ctx.dec_mesh_upload(thin, wl.tets, wl.tags),
